@@ -75,6 +75,7 @@ struct mbs_ctx {
     double snorm_rms = 0.0;  // root mean square over bodies of the Frobenius norm of S
     bool in_solve = false;
     bool df_active = false;
+    bool fx_off = false;  // no memory for the fixed-point kernel's workspace: the other FP64-accurate kernels run
     std::vector<int64_t> off, voff;
     std::vector<int> kb;  // per-body skeleton count
     std::vector<double> skel_world;  // dim * N SoA
@@ -132,8 +133,11 @@ struct mbs_ctx {
 
 namespace {
 
+bool drop_fx(mbs_ctx* c);
+
 void* dalloc(mbs_ctx* c, size_t bytes) {
     if (bytes == 0) bytes = 16;
+    if (c->opt.hbm_budget && c->bytes_held + bytes > c->opt.hbm_budget && drop_fx(c)) return dalloc(c, bytes);
     if (c->opt.hbm_budget && c->bytes_held + bytes > c->opt.hbm_budget)
         throw MbsError{MBS_ERR_NOMEM, "HBM budget exceeded (" + std::to_string(c->bytes_held + bytes) +
                                           " > " + std::to_string(c->opt.hbm_budget) + " bytes)"};
@@ -141,6 +145,7 @@ void* dalloc(mbs_ctx* c, size_t bytes) {
     cudaError_t e = cudaMalloc(&p, bytes);
     if (e != cudaSuccess) {
         cudaGetLastError();
+        if (drop_fx(c)) return dalloc(c, bytes);
         throw MbsError{MBS_ERR_NOMEM, std::string("cudaMalloc(") + std::to_string(bytes) +
                                           "): " + cudaGetErrorString(e)};
     }
@@ -177,6 +182,20 @@ void clear_graphs(mbs_ctx* c) {
     c->graphs.clear();
 }
 
+// The fixed-point kernel's workspace gives way to any other allocation: a
+// context whose memory or budget is exhausted goes on with the other
+// FP64-accurate kernels, which need none.
+bool drop_fx(mbs_ctx* c) {
+    auto it = c->bufs.find("fx_pack");
+    if (it == c->bufs.end() || !it->second.p || c->capturing) return false;
+    clear_graphs(c);
+    if (c->st) cudaStreamSynchronize(c->st);
+    dfree(c, it->second.p);
+    it->second = DevBuf{};
+    c->fx_off = true;
+    return true;
+}
+
 template <typename T>
 T* scratch(mbs_ctx* c, const std::string& name, size_t count) {
     DevBuf& b = c->bufs[name];
@@ -206,6 +225,7 @@ void free_geometry(mbs_ctx* c) {
     c->shapes.clear();
     c->bodies.clear();
     c->built = false;
+    c->fx_off = false;
     c->T = 0;
     c->N = 0;
     c->d_body = nullptr;
@@ -312,10 +332,18 @@ int* split_table(mbs_ctx* c, int ns) {
     return d;
 }
 
-int* split_for(mbs_ctx* c, int64_t ntargets, int* nsplit_out) {
-    const int ns = choose_nsplit(c, ntargets);
-    *nsplit_out = ns;
-    return split_table(c, ns);
+// Workspace of the fixed-point kernel, the default FP64-accurate one
+// (fp64_kernel = 2); null where an option picks another kernel or there is no
+// memory for it.  Taken after every other buffer of a call (see drop_fx).
+void* fx_workspace(mbs_ctx* c, int nrhs) {
+    if (c->opt.fp64_kernel != 2 || c->fx_off) return nullptr;
+    try {
+        return scratch<unsigned char>(c, "fx_pack", fx_pack_bytes(c->dim, c->N, c->T, nrhs));
+    } catch (const MbsError& e) {
+        if (e.st != MBS_ERR_NOMEM) throw;
+        c->fx_off = true;
+        return nullptr;
+    }
 }
 
 GLayout glayout(mbs_ctx* c) {
@@ -534,10 +562,17 @@ void G32(mbs_ctx* c, int nrhs, const float2* x, float2* y) {
     c->last_path = sh.path;
     c->last_nsplit = sh.nsplit;
 }
+// Source splits of the fixed-point kernel: about four rounds of CTAs.
+int fx_nsplit(mbs_ctx* c, int64_t ntargets) {
+    return choose_nsplit(c, ntargets * 256 / fx_tile(ntargets, c->T));
+}
+
 void G64(mbs_ctx* c, int nrhs, const double2* x, double2* y) {
-    int ns;
-    int* sb = split_for(c, c->N, &ns);
-    double2* part = scratch<double2>(c, "part64", (size_t)ns * nrhs * c->N);
+    const bool want_fx = c->opt.fp64_kernel == 2 && !c->fx_off;
+    const int ns64 = choose_nsplit(c, c->N), nsfx = want_fx ? fx_nsplit(c, c->N) : 0;
+    double2* part = scratch<double2>(c, "part64", (size_t)std::max(ns64, nsfx) * nrhs * c->N);
+    int* sb = split_table(c, ns64);
+    int* sbfx = want_fx ? split_table(c, nsfx) : nullptr;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (c->profile && c->capturing) {
         e0 = c->cap_e0;
@@ -547,13 +582,31 @@ void G64(mbs_ctx* c, int nrhs, const double2* x, double2* y) {
         e1 = take_event(c);
         c->ev64.emplace_back(e0, e1);
     }
+    if (void* pack = fx_workspace(c, nrhs)) {
+        launch_G_fx(glayout(c), c->d_centres, c->kappa, c->N, c->d_xw64, c->d_body, nrhs, x, y, part, nsfx, sbfx,
+                    pack, c->st, e0, e1);
+        return;
+    }
     if (c->opt.fp64_kernel == 1 || (c->opt.fp64_kernel == 2 && c->in_solve && c->df_active)) {
         // double-float arithmetic on the FP32 pipe (gdf.cu); the events bracket
         // the kernel passes, not the split reduction, as for the FP64 kernel
-        launch_G_df(glayout(c), c->d_centres, c->kappa, nrhs, x, y, part, ns, sb, c->st, e0, e1);
+        launch_G_df(glayout(c), c->d_centres, c->kappa, nrhs, x, y, part, ns64, sb, c->st, e0, e1);
         return;
     }
-    launch_G_f64(glayout(c), c->kappa, nrhs, x, y, part, ns, sb, c->st, e0, e1);
+    launch_G_f64(glayout(c), c->kappa, nrhs, x, y, part, ns64, sb, c->st, e0, e1);
+}
+
+// Skeleton sums at M targets (tbody nullable: per target a body left out).
+void field64(mbs_ctx* c, int nrhs, int64_t M, const double* pts, const double2* q, double2* u, const int* tbody) {
+    const bool want_fx = c->opt.fp64_kernel == 2 && !c->fx_off;
+    const int ns64 = choose_nsplit(c, M), nsfx = want_fx ? fx_nsplit(c, M) : 0;
+    double2* part = scratch<double2>(c, "part_field", (size_t)std::max(ns64, nsfx) * nrhs * M);
+    int* sb = split_table(c, ns64);
+    int* sbfx = want_fx ? split_table(c, nsfx) : nullptr;
+    if (void* pack = fx_workspace(c, nrhs))
+        launch_G_fx(glayout(c), c->d_centres, c->kappa, M, pts, tbody, nrhs, q, u, part, nsfx, sbfx, pack, c->st);
+    else
+        launch_field_f64(glayout(c), c->kappa, M, pts, nrhs, q, u, part, ns64, sb, c->st, tbody);
 }
 
 // out = x + S G_hat x
@@ -2009,7 +2062,7 @@ mbs_status mbs_solve(mbs_ctx* c, int nrhs, const double* b, double* qhat, mbs_so
         finish_out(c, ox);
         inf.converged = conv ? 1 : 0;
         inf.rel_residual = relmax;
-        inf.fp64_kernel = df ? 1 : 0;
+        inf.fp64_kernel = k64 == 2 && !c->fx_off ? 2 : df ? 1 : 0;
         inf.seconds = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
         if (info) *info = inf;
         if (!conv) {
@@ -2040,10 +2093,7 @@ mbs_status mbs_evaluate_field(mbs_ctx* c, int nrhs, int64_t M, const double* pts
         const double* dp = in_dev_real(c, pts, (size_t)c->dim * M, "io_pts");
         const double2* dq = in_dev(c, qhat, (size_t)c->N * nrhs, "io_q");
         OutBuf ou = out_dev(c, u, (size_t)M * nrhs, "io_u");
-        int ns;
-        int* sb = split_for(c, M, &ns);
-        double2* part = scratch<double2>(c, "part_field", (size_t)ns * nrhs * M);
-        launch_field_f64(glayout(c), c->kappa, M, dp, nrhs, dq, ou.dev, part, ns, sb, c->st);
+        field64(c, nrhs, M, dp, dq, ou.dev, nullptr);
         finish_out(c, ou);
         return MBS_OK;
     });
@@ -2082,11 +2132,8 @@ mbs_status mbs_evaluate_field_near(mbs_ctx* c, int nrhs, int64_t M, const double
         const double2* dq = in_dev(c, qhat, (size_t)c->N * nrhs, "io_q");
         const double2* dm = in_dev(c, qmfs, (size_t)c->Nm * nrhs, "io_qmfs_in");
         OutBuf ou = out_dev(c, u, (size_t)M * nrhs, "io_u");
-        int ns;
-        int* sb = split_for(c, M, &ns);
-        double2* part = scratch<double2>(c, "part_field", (size_t)ns * nrhs * M);
         // skeleton sums of every body but the one whose proxy holds the target ...
-        launch_field_f64(glayout(c), c->kappa, M, dp, nrhs, dq, ou.dev, part, ns, sb, c->st, d_tb);
+        field64(c, nrhs, M, dp, dq, ou.dev, d_tb);
         // ... plus that body's reconstructed MFS sources
         launch_mfs_near(c->dim, M, dp, d_tb, c->d_mfsb, c->kappa, nrhs, dm, c->Nm, ou.dev, c->st);
         finish_out(c, ou);

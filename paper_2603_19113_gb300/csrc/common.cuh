@@ -117,6 +117,25 @@ void launch_G_f64(const GLayout& L, double kappa, int nrhs, const double2* q, do
 void launch_G_df(const GLayout& L, const double* d_centres, double kappa, int nrhs, const double2* q,
                  double2* y, double2* part, int nsplit, const int* d_split_body, cudaStream_t st,
                  cudaEvent_t ev0 = nullptr, cudaEvent_t ev1 = nullptr);
+// FP64-accurate sums in 64-bit fixed point (gfixed.cu): Nt targets (SoA dim x
+// Nt; tbody nullable: per target a body that is left out), q and the sources
+// of L; pack: fx_pack_bytes() of workspace; nsplit source splits for tiles of
+// fx_tile() targets.
+struct FxPacked {
+    int4* q;        // [nrhs][N] entries as integers: re and im, high and low words
+    double* qs;     // [nrhs][T] their scale per body
+    long long* d;   // [dim][N] offsets from the body centre as integers
+    float* rho;     // [T] radius about the centre
+    int* es;        // [T] exponent of the offsets
+};
+size_t fx_pack_bytes(int dim, int64_t N, int T, int nrhs);
+FxPacked fx_packed(void* p, int dim, int64_t N, int T, int nrhs);
+int fx_groups(int64_t Nt, int T);
+int fx_tile(int64_t Nt, int T);
+void launch_G_fx(const GLayout& L, const double* d_centres, double kappa, int64_t Nt, const double* tgt,
+                 const int* tbody, int nrhs, const double2* q, double2* y, double2* part, int nsplit,
+                 const int* d_split_body, void* pack, cudaStream_t st, cudaEvent_t ev0 = nullptr,
+                 cudaEvent_t ev1 = nullptr);
 // y = sum over the nsplit partial sums part[s * len + e], in split order
 // (deterministic); shared by the FP64-accurate G_hat kernels.
 void launch_reduce_splits64(const double2* part, int nsplit, int64_t len, double2* y, cudaStream_t st);
