@@ -122,7 +122,8 @@ void launch_G_df(const GLayout& L, const double* d_centres, double kappa, int nr
 // of L; pack: fx_pack_bytes() of workspace; nsplit source splits for tiles of
 // fx_tile() targets.
 struct FxPacked {
-    int4* q;        // [nrhs][N] entries as integers: re and im, high and low words
+    float4* ql;     // [nrhs][N] entries as integers, high and low words of re and im as floats
+    int2* qh;       // [nrhs][N] the high words of re and im
     double* qs;     // [nrhs][T] their scale per body
     long long* d;   // [dim][N] offsets from the body centre as integers
     float* rho;     // [T] radius about the centre

@@ -5,9 +5,10 @@
 //
 // phi comes from phi_fx.h (72 wide integer multiply-adds a pair in 2D, against
 // about 50 FP64 operations that take 16 times as long each); the product with
-// the right-hand sides is exact to 2^-59 of the largest |q| of a source body,
-// also on the integer multipliers (14 wide multiply-adds a pair and
-// right-hand side), and goes into FP64 sums once per body.
+// the right-hand sides, integers of 60 bits relative to the largest |q| of a
+// source body, takes 4 wide multiply-adds and 8 FP32 ones (the cross terms of
+// high and low words, whose 24 bits end near 2^-56) a pair and right-hand side,
+// and goes into FP64 sums once per round of 64 sources.
 //
 // g_fx_pack_kernel, one CTA per body, turns the offsets from the body's centre
 // and the right-hand sides into integers scaled by the body's own radius and
@@ -26,7 +27,8 @@ __device__ const FxSteps g_fx_steps = fx_steps();
 
 constexpr int FXT = 128;     // threads per CTA
 constexpr int FX_SB = 64;    // sources staged per round
-constexpr int FX_QBITS = 61;  // right-hand sides are integers below 2^61: 64 products stay below 2^62 in an integer sum
+constexpr int FX_QBITS = 60;  // right-hand sides are integers below 2^60: 64 products stay below 2^62 in an integer sum
+constexpr int FX_CROSS = 4;   // sources per FP32 sum of cross terms (below 2^63: its integer part fits 32 bits)
 constexpr int FX_BAD = INT_MIN;  // stored exponent of a body whose values need FP64
 
 __device__ __forceinline__ double fx_block_max(double v, double* s) {
@@ -84,7 +86,8 @@ __global__ void __launch_bounds__(FXT) g_fx_pack_kernel(const int64_t N, const i
         for (int64_t j = j0 + threadIdx.x; j < j1; j += FXT) {
             const double2 v = q[(int64_t)r * N + j];
             const fx2 re = fx_split(out ? 0 : fx_round(v.x * sc)), im = fx_split(out ? 0 : fx_round(v.y * sc));
-            P.q[(int64_t)r * N + j] = make_int4(re.h, re.l, im.h, im.l);
+            P.qh[(int64_t)r * N + j] = make_int2(re.h, im.h);
+            P.ql[(int64_t)r * N + j] = make_float4((float)re.h, (float)re.l, (float)im.h, (float)im.l);
         }
         if (threadIdx.x == 0) P.qs[(int64_t)r * T + b] = fx_exp2(ex + 64 - FX_QBITS);  // of sums kept at 2^-64
     }
@@ -112,7 +115,8 @@ __global__ void __launch_bounds__(FXT, 4)
     constexpr int TG = FXT / SG;
     __shared__ FxEntry s_tab[FX_TAB];
     __shared__ fx_i64 s_d[FX_SB][DIM];
-    __shared__ int4 s_q[FX_SB][NR];
+    __shared__ int2 s_qh[FX_SB][NR];    // high words of re q, im q
+    __shared__ float4 s_ql[FX_SB][NR];  // re high, re low, im high, im low as floats
     __shared__ double2 s_acc[NR][FXT];
     const int tid = threadIdx.x, grp = tid / TG;
     for (int k = tid; k < FX_TAB; k += FXT) s_tab[k] = g_fx_steps.e[k];
@@ -139,9 +143,24 @@ __global__ void __launch_bounds__(FXT, 4)
         }
         const bool fast = act && es != FX_BAD && fx_body<DIM>(kap, D, Dl, sqrtf(R2), P.rho[sb], es, B, scale);
         fx_i64 ar[NR], ai[NR];
+        float mr[NR], mi[NR];
 #pragma unroll
-        for (int r = 0; r < NR; ++r) ar[r] = ai[r] = 0;
+        for (int r = 0; r < NR; ++r) {
+            ar[r] = ai[r] = 0;
+            mr[r] = mi[r] = 0.f;
+        }
+        // the cross terms into the integer sums, every few sources: their FP32
+        // sum rounds at 2^-24 of its own size
+        auto carry = [&]() {
+#pragma unroll
+            for (int r = 0; r < NR; ++r) {
+                ar[r] += __float2int_rn(mr[r] * 0x1p-32f);
+                ai[r] += __float2int_rn(mi[r] * 0x1p-32f);
+                mr[r] = mi[r] = 0.f;
+            }
+        };
         auto flush = [&]() {
+            carry();
 #pragma unroll
             for (int r = 0; r < NR; ++r)
                 if (r0 + r < nrhs) {
@@ -159,7 +178,9 @@ __global__ void __launch_bounds__(FXT, 4)
             for (int k = tid; k < n * DIM; k += FXT) s_d[k % n][k / n] = P.d[(int64_t)(k / n) * N + jc + k % n];
             for (int k = tid; k < n * NR; k += FXT) {
                 const int r = k / n, j = k - r * n;
-                s_q[j][r] = r0 + r < nrhs ? P.q[(int64_t)(r0 + r) * N + jc + j] : make_int4(0, 0, 0, 0);
+                const bool in = r0 + r < nrhs;
+                s_qh[j][r] = in ? P.qh[(int64_t)(r0 + r) * N + jc + j] : make_int2(0, 0);
+                s_ql[j][r] = in ? P.ql[(int64_t)(r0 + r) * N + jc + j] : make_float4(0.f, 0.f, 0.f, 0.f);
             }
             __syncthreads();
             const int part_n = (n + SG - 1) / SG;
@@ -179,17 +200,21 @@ __global__ void __launch_bounds__(FXT, 4)
                         pr = fx_round(p.x / scale);
                         pi = fx_round(p.y / scale);
                     }
+                    // high x high words exactly on the integer multipliers; the
+                    // cross terms, 2^-32 of them, in FP32 beside them
                     const fx2 a = fx_split(pr), b = fx_split(pi);
-                    const int nh = -b.h, nl = -b.l;
+                    const int nh = -b.h;
+                    const float ah = (float)a.h, al = (float)a.l, bh = (float)b.h, bl = (float)b.l;
 #pragma unroll
                     for (int r = 0; r < NR; ++r) {
-                        const int4 v = s_q[j][r];
-                        // rounded, not cut: a floor would add up over the sources
-                        const fx_i64 mr = fx_madw(a.h, v.y, fx_madw(a.l, v.x, fx_madw(nh, v.w, fx_madw(nl, v.z, 0x80000000ll))));
-                        const fx_i64 mi = fx_madw(a.h, v.w, fx_madw(a.l, v.z, fx_madw(b.h, v.y, fx_madw(b.l, v.x, 0x80000000ll))));
-                        ar[r] = fx_madw(a.h, v.x, fx_madw(nh, v.z, fx_madw(fx_hi(mr), 1, ar[r])));
-                        ai[r] = fx_madw(a.h, v.z, fx_madw(b.h, v.x, fx_madw(fx_hi(mi), 1, ai[r])));
+                        const int2 v = s_qh[j][r];
+                        const float4 w = s_ql[j][r];
+                        ar[r] = fx_madw(a.h, v.x, fx_madw(nh, v.y, ar[r]));
+                        ai[r] = fx_madw(a.h, v.y, fx_madw(b.h, v.x, ai[r]));
+                        mr[r] = fmaf(ah, w.y, fmaf(al, w.x, fmaf(-bh, w.w, fmaf(-bl, w.z, mr[r]))));
+                        mi[r] = fmaf(ah, w.w, fmaf(al, w.z, fmaf(bh, w.y, fmaf(bl, w.x, mi[r]))));
                     }
+                    if ((j - k0) % FX_CROSS == FX_CROSS - 1) carry();
                 }
                 flush();
             } else if (act) {
@@ -248,15 +273,17 @@ void launch_fx(const GLayout& L, const double* centres, const FxKappa& k, int64_
 }  // namespace
 
 size_t fx_pack_bytes(int dim, int64_t N, int T, int nrhs) {
-    return (size_t)N * nrhs * sizeof(int4) + (size_t)nrhs * T * sizeof(double) +
+    return (size_t)N * nrhs * (sizeof(int2) + sizeof(float4)) + (size_t)nrhs * T * sizeof(double) +
            (size_t)dim * N * sizeof(fx_i64) + (size_t)T * (sizeof(float) + sizeof(int));
 }
 
 FxPacked fx_packed(void* p, int dim, int64_t N, int T, int nrhs) {
     unsigned char* c = static_cast<unsigned char*>(p);
     FxPacked P;
-    P.q = reinterpret_cast<int4*>(c);
-    c += (size_t)N * nrhs * sizeof(int4);
+    P.ql = reinterpret_cast<float4*>(c);
+    c += (size_t)N * nrhs * sizeof(float4);
+    P.qh = reinterpret_cast<int2*>(c);
+    c += (size_t)N * nrhs * sizeof(int2);
     P.qs = reinterpret_cast<double*>(c);
     c += (size_t)nrhs * T * sizeof(double);
     P.d = reinterpret_cast<fx_i64*>(c);

@@ -160,6 +160,7 @@ struct FxBody {
     fx2 K;          // kappa 2^e / (2 pi), as a mantissa at 2^62
     int ksh;        // left shift of r K to turns at 2^64
     fx2 Ki;         // 2D: 1 / (kappa 2^e) at 2^66
+    int up;         // left shift that brings the largest amplitude near 2^61
 };
 
 // Lengths below 2^-4 of 2^e would leave the integer formats: such bodies
@@ -176,7 +177,10 @@ FX_HD bool fx_body(const FxKappa& k, const double* D, const double* Dl, double R
     if (!(rmax > 1e-90 && rmax < 1e90)) return false;
     int e = fx_exponent(rmax);
     if (e < es) e = es;
-    if (!((R - rho) >= FX_RMIN * fx_exp2(e))) return false;
+    const double rmin = (R - rho) * (1.0 - 1e-6);
+    if (!(rmin >= FX_RMIN * fx_exp2(e))) return false;
+    const int j = e + 1 - fx_exponent(rmin);  // r / 2^e >= 2^-j, 1 <= j <= 4
+    b.up = DIM == 2 ? (j <= 1 ? 2 : j <= 3 ? 1 : 0) : 5 - j;
     const int ksh = k.kturn_e + e + 4;  // (2^62 2^62 2^-64) 2^ksh = 2^64 / 2^(kturn_e + e)
     if (ksh < -30 || ksh > 40) return false;  // kappa 2^e between 2^-34 and 2^36 turns
     if (DIM == 2) {
@@ -191,20 +195,24 @@ FX_HD bool fx_body(const FxKappa& k, const double* D, const double* Dl, double R
     b.sh = e - es > 63 ? 63 : e - es;
     b.ksh = ksh > 0 ? ksh : 0;
     b.K = fx_split(ksh < 0 ? k.kturn62 >> -ksh : k.kturn62);
-    // fx_phi returns the amplitude relative to that at r = 2^e times 2^56 (2D) or 2^54 (3D)
+    // fx_phi returns the amplitude relative to that at r = 2^e times 2^(56 + up) (2D) or 2^(54 + up) (3D)
     if (DIM == 2)
-        scale = k.amp * ((e & 1) ? 0.70710678118654752440 * fx_exp2(-(e - 1) / 2 - 56) : fx_exp2(-e / 2 - 56));
+        scale = k.amp * ((e & 1) ? 0.70710678118654752440 * fx_exp2(-(e - 1) / 2 - 56 - b.up) : fx_exp2(-e / 2 - 56 - b.up));
     else
-        scale = k.amp * fx_exp2(-e - 54);
+        scale = k.amp * fx_exp2(-e - 54 - b.up);
     return true;
 }
 
-// Polynomials in u (|u| <= 1, at 2^62) with coefficients at 2^62, highest first
-FX_HD fx_i64 fx_horner(const fx_i64* c, int deg, fx2 u) {
-    fx_i64 p = c[0];
-#pragma unroll 1
-    for (int k = 1; k <= deg; ++k) p = (fx_mulhi(fx_split(p), u) << 2) + c[k];
-    return p;
+// Two polynomials in u (|u| <= 1, at 2^62) with coefficients at 2^62, highest
+// first; side by side, so that each hides the other's latency
+FX_HD void fx_horner2(const fx_i64* cf, const fx_i64* cg, int deg, fx2 u, fx_i64& f, fx_i64& g) {
+    f = cf[0];
+    g = cg[0];
+#pragma unroll 2
+    for (int k = 1; k <= deg; ++k) {
+        f = (fx_mulhi(fx_split(f), u) << 2) + cf[k];
+        g = (fx_mulhi(fx_split(g), u) << 2) + cg[k];
+    }
 }
 
 #if defined(__CUDACC__)
@@ -268,7 +276,7 @@ FX_HD void fx_cis(fx_u64 theta, const FxEntry* tab, fx_i64& dc, fx_i64& ds) {
 }
 
 // phi for one source at stored offset dj: the integers re, im, with
-// phi = scale (re + i im) and |re|, |im| < 2^59.  2D: false below kappa r = 4
+// phi = scale (re + i im) and |re|, |im| <= 2^59.  2D: false below kappa r = 4
 // (the caller evaluates those pairs in FP64).  tab: cos and sin of k / 1024 turns.
 template <int DIM>
 FX_HD bool fx_phi(const FxBody<DIM>& b, const fx_i64* dj, const FxEntry* tab, fx_i64& re, fx_i64& im) {
@@ -289,9 +297,10 @@ FX_HD bool fx_phi(const FxBody<DIM>& b, const fx_i64* dj, const FxEntry* tab, fx
     const float r0f = af * y;
     const int r0 = fx_rint(r0f * 0x1p31f);
     const fx_i64 eps = fx_madw(-r0, r0, A);
-    const int c = fx_rint((float)(int)(eps >> 20) * (y * 256.0f));  // at 2^51
-    const fx_i64 t = fx_madw(-fx_hi(fx_mulw(c, c)), 4096, fx_madw(-2 * c, r0, eps << 20));  // at 2^82
-    const int c2 = fx_rint((float)(int)(t >> 14) * (y * 0x1p-7f));  // at 2^62
+    const float cf = (float)(int)(eps >> 20) * (y * 256.0f);
+    const int c = fx_rint(cf);                               // at 2^51
+    const fx_i64 t = fx_madw(-2 * c, r0, eps << 20);         // at 2^82, c^2 still to be taken off
+    const int c2 = fx_rint(fmaf(cf, cf * -0x1p-34f, (float)(int)(t >> 14)) * (y * 0x1p-7f));  // at 2^62
     const fx_i64 cc = fx_madw(c, 2048, c2);
     const fx_i64 r = ((fx_i64)r0 << 31) + cc;
     // 1 / sqrt(r) = q0 (1 - w)^{-1/2}, w = 1 - q0^2 r: the residual of q0^2 r0
@@ -305,7 +314,7 @@ FX_HD bool fx_phi(const FxBody<DIM>& b, const fx_i64* dj, const FxEntry* tab, fx
     const fx_i64 w = (w0 >> 8) - fx_madw(Qs.h, C32, fx_hi(fx_mulw(Qs.l, C32)));
     const int w32 = (int)(w >> 25);               // at 2^50
     const int w2 = fx_hi(fx_mulw(w32, w32));      // w^2 at 2^68
-    fx_i64 amp;                                   // 2D at 2^58, 3D at 2^56
+    fx_i64 amp;                                   // 2D at 2^(58 + up), 3D at 2^(56 + up)
     fx_u64 theta;                                 // turns at 2^64
     {
         const fx_i64 p = fx_mulhi(fx_split(r), b.K);
@@ -314,7 +323,7 @@ FX_HD bool fx_phi(const FxBody<DIM>& b, const fx_i64* dj, const FxEntry* tab, fx
     if (DIM == 3) {
         const fx2 ws = fx_split(w);
         const fx_i64 qw = fx_mulhi(Qs, ws) + (fx_mulw(Qs.h, w2) >> 25);  // Q (w + w^2) at 2^67
-        amp = (fx_i64)Q + (qw >> 11);
+        amp = ((fx_i64)Q + (qw >> 11)) << b.up;
     } else {
         const fx_i64 rinv =
             (fx_i64)Q + (fx_madw(Qs.h, w32, fx_hi(fx_mulw(Qs.l, w32)) + (fx_mulw(Qs.h, w2) >> 18)) >> 18);
@@ -331,12 +340,12 @@ FX_HD bool fx_phi(const FxBody<DIM>& b, const fx_i64* dj, const FxEntry* tab, fx
                 (fx_mulhi(ss, fx_split(5871781006564002453ll)) << 2);  // 1 / (16 pi) at 2^68
         } else if (s <= (fx_i64)1 << 54) {  // kappa r >= 16: u = 32 s - 1
             const fx2 u = fx_split((s << 9) - ((fx_i64)1 << 62));
-            f1 = fx_horner(c_fx16F.c, MBS_F64_X16_DEG, u);
-            g = fx_horner(c_fx16G.c, MBS_F64_X16_DEG, u) << 2;
+            fx_horner2(c_fx16F.c, c_fx16G.c, MBS_F64_X16_DEG, u, f1, g);
+            g <<= 2;
         } else if (s <= (fx_i64)1 << 56) {  // kappa r >= 4: u = 8 s - 1
             const fx2 u = fx_split((s << 7) - ((fx_i64)1 << 62));
-            f1 = fx_horner(c_fx4F.c, MBS_F64_X4_DEG, u);
-            g = fx_horner(c_fx4G.c, MBS_F64_X4_DEG, u) << 2;
+            fx_horner2(c_fx4F.c, c_fx4G.c, MBS_F64_X4_DEG, u, f1, g);
+            g <<= 2;
         } else {
             re = im = 0;
             return false;
@@ -346,7 +355,7 @@ FX_HD bool fx_phi(const FxBody<DIM>& b, const fx_i64* dj, const FxEntry* tab, fx
         const fx_i64 m = ((fx_i64)1 << 62) + (w >> 14) + ((3 * w2) >> 9) + f1 +
                          (fx_mulw(w32, (int)(f1 >> 24)) >> 27);
         const fx2 ms = fx_split(m);
-        amp = fx_madw(q0, ms.h, fx_hi(fx_mulw(q0, ms.l)));
+        amp = fx_madw(q0 << b.up, ms.h, fx_hi(fx_mulw(q0 << b.up, ms.l)));
     }
     fx_i64 dc, ds;
     fx_cis(theta, tab, dc, ds);
