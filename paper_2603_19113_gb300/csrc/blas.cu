@@ -150,16 +150,18 @@ __device__ __forceinline__ T warp_sum_t(T v) {
 
 // partial[(i*nrhs + r) * nblk + blk] = sum over the block's slice of conj(basis_{i,r}) . w_r
 // for every i < nvec.  The block keeps its slice of w_r in registers and walks
-// the basis vectors; per-thread sums are in the vector's precision, the
-// cross-warp sums in FP64 and in a fixed order (bitwise reproducible).
+// `per` of the basis vectors (blockIdx.z); per-thread sums are in the vector's
+// precision, the cross-warp sums in FP64 and in a fixed order (bitwise
+// reproducible, whatever `per` is).
 template <typename V>
 __global__ void __launch_bounds__(256) dots_kernel(const V* __restrict__ basis, const int nvec,
                                                    const V* __restrict__ w, const int64_t N,
                                                    const int nrhs, double2* __restrict__ partial,
-                                                   const int nblk) {
+                                                   const int nblk, const int per) {
     using T = typename Acc<V>::T;
-    extern __shared__ double2 s_acc[];  // [warp][nvec]
+    extern __shared__ double2 s_acc[];  // [warp][per]
     const int r = blockIdx.y, blk = blockIdx.x;
+    const int i0 = blockIdx.z * per, n_i = min(per, nvec - i0);
     const int64_t chunk = (N + nblk - 1) / nblk;
     const int64_t n0 = (int64_t)blk * chunk, n1 = min(N, n0 + chunk);
     V wv[DOT_E];
@@ -171,8 +173,9 @@ __global__ void __launch_bounds__(256) dots_kernel(const V* __restrict__ basis, 
         wv[e] = n < n1 ? w[(int64_t)r * N + n] : z;
     }
     const int warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
-    for (int i = 0; i < nvec; ++i) {
-        const V* __restrict__ vb = basis + ((int64_t)i * nrhs + r) * N;
+#pragma unroll 2
+    for (int i = 0; i < n_i; ++i) {
+        const V* __restrict__ vb = basis + ((int64_t)(i0 + i) * nrhs + r) * N;
         T sx = T(0), sy = T(0);
 #pragma unroll
         for (int e = 0; e < DOT_E; ++e) {
@@ -185,14 +188,14 @@ __global__ void __launch_bounds__(256) dots_kernel(const V* __restrict__ basis, 
         }
         sx = warp_sum_t(sx);
         sy = warp_sum_t(sy);
-        if ((threadIdx.x & 31) == 0) s_acc[(int64_t)warp * nvec + i] = make_double2(sx, sy);
+        if ((threadIdx.x & 31) == 0) s_acc[(int64_t)warp * per + i] = make_double2(sx, sy);
     }
     __syncthreads();
     // warps are summed in a fixed order: the result does not depend on scheduling
-    for (int i = threadIdx.x; i < nvec; i += blockDim.x) {
+    for (int i = threadIdx.x; i < n_i; i += blockDim.x) {
         double2 s = s_acc[i];
-        for (int wi = 1; wi < nwarp; ++wi) s = cadd(s, s_acc[(int64_t)wi * nvec + i]);
-        partial[((int64_t)i * nrhs + r) * nblk + blk] = s;
+        for (int wi = 1; wi < nwarp; ++wi) s = cadd(s, s_acc[(int64_t)wi * per + i]);
+        partial[((int64_t)(i0 + i) * nrhs + r) * nblk + blk] = s;
     }
 }
 
@@ -241,6 +244,7 @@ __global__ void __launch_bounds__(256) update_kernel(const V* __restrict__ basis
          n += (int64_t)gridDim.x * blockDim.x) {
         V o = w[(int64_t)r * N + n];
         T ax = o.x, ay = o.y;
+#pragma unroll 8
         for (int i = 0; i < nvec; ++i) {
             const V v = basis[((int64_t)i * nrhs + r) * N + n];
             const V c = s_h[i];
@@ -964,14 +968,19 @@ void launch_dots(const V* basis, int nvec, const V* w, int64_t N, int nrhs, doub
     if (nvec == 0) return;
     if ((int64_t)nblk * 256 * DOT_E < N)
         throw MbsError{MBS_ERR_ARG, "launch_dots: too few blocks for the vector length"};
-    dim3 g((unsigned)nblk, (unsigned)nrhs);
-    const size_t sm = (size_t)nvec * (256 / 32) * sizeof(double2);
-    if (sm > 227 * 1024) throw MbsError{MBS_ERR_ARG, "launch_dots: too many basis vectors"};
-    if (sm > 48 * 1024)
-        MBS_CUDA_TRY(cudaFuncSetAttribute(dots_kernel<V>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)sm));
-    dots_kernel<V><<<g, 256, sm, st>>>(basis, nvec, w, N, nrhs, scratch, nblk);
+    if ((size_t)nvec * (256 / 32) * sizeof(double2) > 227 * 1024)
+        throw MbsError{MBS_ERR_ARG, "launch_dots: too many basis vectors"};
+    // Vectors per CTA: as many as keep about four CTAs on every SM.  At N = 640
+    // and one right-hand side three CTAs walked all of up to 60 vectors (39 us);
+    // one CTA per vector takes 4 us.
+    const int64_t slots = 4LL * mbs_num_sms();
+    const int per = (int)std::min<int64_t>(std::max<int64_t>(1, ((int64_t)nvec * nblk * nrhs + slots - 1) / slots), 256);
+    const dim3 g((unsigned)nblk, (unsigned)nrhs, (unsigned)((nvec + per - 1) / per));
+    const size_t sm = (size_t)per * (256 / 32) * sizeof(double2);
+    // one block: its sums are the results
+    dots_kernel<V><<<g, 256, sm, st>>>(basis, nvec, w, N, nrhs, nblk == 1 ? out : scratch, nblk, per);
     MBS_CHECK_LAUNCH();
+    if (nblk == 1) return;
     dots_finish_kernel<<<nblocks((int64_t)nvec * nrhs * 32, 256), 256, 0, st>>>(scratch, nvec * nrhs, nblk, out);
     MBS_CHECK_LAUNCH();
 }

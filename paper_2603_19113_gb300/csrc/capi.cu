@@ -634,8 +634,11 @@ void apply_op<double2>(mbs_ctx* c, int nrhs, const double2* x, double2* out) {
 
 // Blocks per RHS of the dot-product kernel: each block covers at most 2048
 // rows (its slice of w stays in registers); aim at ~4 blocks per SM overall.
+// Vectors that fit one block take one, which leaves out the pass that adds the
+// blocks' sums (3 us of a 10-body solve's step, three times).
 int dot_blocks(int64_t N, int nrhs) {
     const int64_t minb = (N + 2047) / 2048;
+    if (minb <= 1) return 1;
     const int64_t want = (4LL * mbs_num_sms() + nrhs - 1) / nrhs;
     const int64_t maxb = (N + 255) / 256;
     return (int)std::max<int64_t>(1, std::max(minb, std::min(want, maxb)));
