@@ -1634,6 +1634,7 @@ void build(mbs_ctx* c, int nshapes, const mbs_shape* shapes, int nbodies, const 
             J.permB = (int*)talloc(sizeof(int) * s.m);
             J.diagB = (double2*)talloc(sizeof(double2) * std::min(s.p, s.m));
             J.permA = (int*)talloc(sizeof(int) * s.n);
+            J.ctl = (int*)talloc(sizeof(int) * 4);
             J.diagA = (double2*)talloc(sizeof(double2) * s.n);
             s.JA = galloc<double2>(c, (size_t)s.n * s.n);
             s.FA = galloc<double2>(c, (size_t)s.n * s.n);

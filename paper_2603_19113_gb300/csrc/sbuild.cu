@@ -65,6 +65,28 @@ constexpr double B_QR_CUT = 10.0;
 // warps of the CTA (the block size is chosen at launch)
 __device__ __forceinline__ int nwarps() { return (int)(blockDim.x >> 5); }
 
+// The CTAs that build one shape together: one, or a thread-block cluster when
+// there are fewer shapes than SMs.  Columns and entries are dealt out over the
+// team's warps and threads; what decides the course of a factorisation is
+// computed by every CTA from the same values (or by CTA 0 alone), and every sum
+// is formed by one warp or one CTA in the same order as with one CTA, so the
+// results do not depend on the team's size.
+struct Team {
+    int rank, size;
+    __device__ __forceinline__ int warp() const { return rank * nwarps() + (int)(threadIdx.x >> 5); }
+    __device__ __forceinline__ int warps() const { return size * nwarps(); }
+    __device__ __forceinline__ int64_t thread() const { return (int64_t)rank * blockDim.x + threadIdx.x; }
+    __device__ __forceinline__ int64_t threads() const { return (int64_t)size * blockDim.x; }
+    // all writes of the team to global memory before the call are visible after it
+    __device__ __forceinline__ void sync() const {
+        __syncthreads();
+        if (size > 1) {
+            __threadfence();
+            asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+        }
+    }
+};
+
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -136,9 +158,9 @@ __device__ int block_argmin(int key, int idx, Red& r) {
 }
 
 template <int DIM>
-__device__ void fill_kernel_matrix(double2* M, int ld, const double* T, int nt, const double* S,
+__device__ void fill_kernel_matrix(const Team& tm, double2* M, int ld, const double* T, int nt, const double* S,
                                    int ns, double kappa) {
-    for (int64_t e = threadIdx.x; e < (int64_t)nt * ns; e += blockDim.x) {
+    for (int64_t e = tm.thread(); e < (int64_t)nt * ns; e += tm.threads()) {
         const int i = (int)(e % nt), j = (int)(e / nt);
         double r2 = 0.0;
 #pragma unroll
@@ -154,10 +176,11 @@ __device__ void fill_kernel_matrix(double2* M, int ld, const double* T, int nt, 
 // ld): the unit reflector v of column j (rows j..rows-1) replaces the column
 // there (H = I - 2 v v^H), diag[j] = R_jj, and H is applied to columns
 // j+1 .. ntot-1 (one warp per column).  With nrm2 given, the squared norms of
-// rows j+1.. of columns j+1 .. ncols-1 are refreshed in full.
-__device__ void householder_step(double2* A, int ld, int rows, int j, int ncols, int ntot,
+// rows j+1.. of columns j+1 .. ncols-1 are refreshed in full.  Every CTA of the
+// team forms the reflector; CTA 0 stores it once all have read the column.
+__device__ void householder_step(const Team& tm, double2* A, int ld, int rows, int j, int ncols, int ntot,
                                  double2* diag, double* nrm2, double2* s_v, Red& red) {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31;
     double2* cj = A + (int64_t)j * ld;
     double sl = 0.0;
     for (int i = j + threadIdx.x; i < rows; i += blockDim.x) sl += cabs2(cj[i]);
@@ -172,13 +195,11 @@ __device__ void householder_step(double2* A, int ld, int rows, int j, int ncols,
     const double inv = nv2 > 0.0 ? 1.0 / sqrt(nv2) : 0.0;
     __syncthreads();
     for (int i = j + threadIdx.x; i < rows; i += blockDim.x) {
-        const double2 v = (i == j) ? cscale(v0, inv) : cscale(cj[i], inv);
-        s_v[i - j] = v;
-        cj[i] = v;
+        s_v[i - j] = (i == j) ? cscale(v0, inv) : cscale(cj[i], inv);
     }
-    if (threadIdx.x == 0) diag[j] = alpha;
+    if (tm.rank == 0 && threadIdx.x == 0) diag[j] = alpha;
     __syncthreads();
-    for (int c = j + 1 + w; c < ntot; c += nwarps()) {
+    for (int c = j + 1 + tm.warp(); c < ntot; c += tm.warps()) {
         double2* cc = A + (int64_t)c * ld;
         double2 d = make_double2(0.0, 0.0);
         for (int i = j + lane; i < rows; i += 32) d = cfmac(s_v[i - j], cc[i], d);
@@ -195,7 +216,9 @@ __device__ void householder_step(double2* A, int ld, int rows, int j, int ncols,
             if (lane == 0) nrm2[c] = s;
         }
     }
-    __syncthreads();
+    tm.sync();
+    if (tm.rank == 0)
+        for (int i = j + threadIdx.x; i < rows; i += blockDim.x) cj[i] = s_v[i - j];
 }
 
 // One-sided Jacobi (Hestenes 1958) on the r columns of X (rows x r, leading
@@ -203,74 +226,148 @@ __device__ void householder_step(double2* A, int ld, int rows, int j, int ncols,
 // is orthogonal to tol relative to the product of their norms; X J = W with
 // orthogonal columns, J (r x r, leading dimension ldj, starts as I)
 // accumulating the rotations.  Pairs are taken in round-robin tournament
-// order, so every round rotates r/2 disjoint pairs, one warp per pair; the
-// result does not depend on the warp schedule.  Returns the sweeps run
-// (maxsweep + 1 if the last one still rotated).
-__device__ int cta_jacobi(double2* X, int ldx, int rows, int r, double2* Jm, int ldj, double tol,
-                          int maxsweep, int* s_flag) {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+// order, so every round rotates r/2 disjoint pairs; the result does not depend
+// on how they are dealt out.  Returns the sweeps run (maxsweep + 1 if the last
+// one still rotated).
+//
+// The FP64 pipe bounds this (a warp instruction takes 16 clocks of the SM
+// whatever its lanes do), and of the ~230 FP64 instructions that a pair of 64
+// rows took when one warp did all of it, 150 were the angle's square roots,
+// divisions and hypotenuses, the same in all lanes.  So a round has three parts:
+// warps sum the three products of up to four pairs at a time (the 16 partial
+// sums of a lane halve in number while they are added, 16 additions instead of
+// 80, in the same tree); one thread per pair finds the angle; warps rotate.
+// The phase for 3 shapes of 64 MFS sources: 28.1 ms to 6.3 ms with 8 CTAs a
+// shape; for 300 shapes of 35 to 105, one CTA each: 202 ms to 106 ms.
+constexpr int JP = 256;  // pairs in flight (larger rounds are taken in parts)
+
+struct Rot {
+    double cs, sn, px, py;
+    int on, i, j;
+};
+
+struct JacobiShared {
+    double sums[JP][4];  // |x_i|^2, |x_j|^2, re and im of x_i^H x_j
+    Rot rot[JP];
+};
+
+__device__ __forceinline__ void jacobi_pair(int pi, int rho, int re, int& i, int& j) {
+    if (pi == 0) {
+        i = rho;
+        j = re - 1;
+    } else {
+        i = (rho + pi) % (re - 1);
+        j = (rho - pi + re - 1) % (re - 1);
+    }
+    if (i > j) {
+        const int t = i;
+        i = j;
+        j = t;
+    }
+}
+
+__device__ int cta_jacobi(const Team& tm, double2* X, int ldx, int rows, int r, double2* Jm, int ldj, double tol,
+                          int maxsweep, int* flag, JacobiShared& sh) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = nwarps();
     const int re = r + (r & 1);  // with a dummy column when r is odd
     const int half = re / 2;
+    // this CTA's pairs of a round: a contiguous part of them
+    const int per = (half + tm.size - 1) / tm.size;
+    const int p0 = min(half, tm.rank * per), p1 = min(half, p0 + per);
     for (int sweep = 0; sweep < maxsweep; ++sweep) {
-        if (threadIdx.x == 0) *s_flag = 0;
-        __syncthreads();
+        if (tm.rank == 0 && threadIdx.x == 0) flag[sweep & 1] = 0;
+        tm.sync();
         for (int rho = 0; rho < re - 1; ++rho) {
-            for (int pi = w; pi < half; pi += nwarps()) {
-                int i, j;
-                if (pi == 0) {
-                    i = rho;
-                    j = re - 1;
-                } else {
-                    i = (rho + pi) % (re - 1);
-                    j = (rho - pi + re - 1) % (re - 1);
+            for (int q0 = p0; q0 < p1; q0 += JP) {
+                const int np = min(JP, p1 - q0);
+                for (int g = 4 * w; g < np; g += 4 * nw) {
+                    const double2 *xi[4], *xj[4];
+                    double v[16];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        int i = 0, j = 0;
+                        const bool in = g + u < np;
+                        if (in) jacobi_pair(q0 + g + u, rho, re, i, j);
+                        xi[u] = in && j < r ? X + (int64_t)i * ldx : nullptr;
+                        xj[u] = X + (int64_t)(j < r ? j : 0) * ldx;
+                        v[4 * u] = v[4 * u + 1] = v[4 * u + 2] = v[4 * u + 3] = 0.0;
+                    }
+                    for (int l = lane; l < rows; l += 32)
+#pragma unroll
+                        for (int u = 0; u < 4; ++u)
+                            if (xi[u]) {
+                                const double2 a = xi[u][l], b = xj[u][l];
+                                v[4 * u] = abs2_acc(a, v[4 * u]);
+                                v[4 * u + 1] = abs2_acc(b, v[4 * u + 1]);
+                                const double2 c = cfmac(a, b, make_double2(v[4 * u + 2], v[4 * u + 3]));
+                                v[4 * u + 2] = c.x;
+                                v[4 * u + 3] = c.y;
+                            }
+#pragma unroll
+                    for (int n = 16, o = 16; n > 1; n >>= 1, o >>= 1) {
+                        const bool up = (lane & o) != 0;
+#pragma unroll
+                        for (int k = 0; k < n / 2; ++k) {
+                            const double keep = up ? v[k + n / 2] : v[k], send = up ? v[k] : v[k + n / 2];
+                            v[k] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+                        }
+                    }
+                    v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+                    // lanes 2 k and 2 k + 1 hold value k % 4 of pair k / 4
+                    if (!(lane & 1) && g + (lane >> 3) < np) sh.sums[g + (lane >> 3)][(lane >> 1) & 3] = v[0];
                 }
-                if (i > j) {
-                    const int t = i;
-                    i = j;
-                    j = t;
+                __syncthreads();
+                for (int q = threadIdx.x; q < np; q += blockDim.x) {
+                    Rot R;
+                    R.on = 0;
+                    jacobi_pair(q0 + q, rho, re, R.i, R.j);
+                    if (R.j < r) {
+                        const double a = sh.sums[q][0], b = sh.sums[q][1];
+                        const double2 c = make_double2(sh.sums[q][2], sh.sums[q][3]);
+                        const double ac = sqrt(cabs2(c));
+                        if (!(!(ac > 0.0) || ac <= tol * sqrt(a) * sqrt(b))) {
+                            // x_j' = e^{-i arg c} x_j makes the pair's inner product real and
+                            // positive; then the real rotation with t = tan(theta) the
+                            // smaller root of t^2 + 2 zeta t - 1 = 0
+                            R.on = 1;
+                            R.px = c.x / ac;
+                            R.py = -c.y / ac;
+                            const double zeta = (b - a) / (2.0 * ac);
+                            const double t = copysign(1.0, zeta) / (fabs(zeta) + hypot(1.0, zeta));
+                            R.cs = 1.0 / hypot(1.0, t);
+                            R.sn = R.cs * t;
+                            flag[sweep & 1] = 1;
+                        }
+                    }
+                    sh.rot[q] = R;
                 }
-                if (j >= r) continue;
-                double2* xi = X + (int64_t)i * ldx;
-                double2* xj = X + (int64_t)j * ldx;
-                double a = 0.0, b = 0.0;
-                double2 c = make_double2(0.0, 0.0);
-                for (int l = lane; l < rows; l += 32) {
-                    const double2 u = xi[l], v = xj[l];
-                    a = abs2_acc(u, a);
-                    b = abs2_acc(v, b);
-                    c = cfmac(u, v, c);
+                __syncthreads();
+                for (int q = w; q < np; q += nw) {
+                    const Rot R = sh.rot[q];
+                    if (!R.on) continue;
+                    const double cs = R.cs, sn = R.sn;
+                    const double2 ph = make_double2(R.px, R.py);
+                    double2* xi = X + (int64_t)R.i * ldx;
+                    double2* xj = X + (int64_t)R.j * ldx;
+                    for (int l = lane; l < rows; l += 32) {
+                        const double2 u = xi[l], v = cmul(ph, xj[l]);
+                        xi[l] = make_double2(cs * u.x - sn * v.x, cs * u.y - sn * v.y);
+                        xj[l] = make_double2(sn * u.x + cs * v.x, sn * u.y + cs * v.y);
+                    }
+                    double2* ji = Jm + (int64_t)R.i * ldj;
+                    double2* jj = Jm + (int64_t)R.j * ldj;
+                    for (int l = lane; l < r; l += 32) {
+                        const double2 u = ji[l], v = cmul(ph, jj[l]);
+                        ji[l] = make_double2(cs * u.x - sn * v.x, cs * u.y - sn * v.y);
+                        jj[l] = make_double2(sn * u.x + cs * v.x, sn * u.y + cs * v.y);
+                    }
                 }
-                a = warp_sum(a);
-                b = warp_sum(b);
-                c = warp_sum2(c);
-                const double ac = sqrt(cabs2(c));
-                if (!(ac > 0.0) || ac <= tol * sqrt(a) * sqrt(b)) continue;
-                if (lane == 0) *s_flag = 1;
-                // x_j' = e^{-i arg c} x_j makes the pair's inner product real and
-                // positive; then the real rotation with t = tan(theta) the
-                // smaller root of t^2 + 2 zeta t - 1 = 0
-                const double2 ph = make_double2(c.x / ac, -c.y / ac);
-                const double zeta = (b - a) / (2.0 * ac);
-                const double t = copysign(1.0, zeta) / (fabs(zeta) + hypot(1.0, zeta));
-                const double cs = 1.0 / hypot(1.0, t);
-                const double sn = cs * t;
-                for (int l = lane; l < rows; l += 32) {
-                    const double2 u = xi[l], v = cmul(ph, xj[l]);
-                    xi[l] = make_double2(cs * u.x - sn * v.x, cs * u.y - sn * v.y);
-                    xj[l] = make_double2(sn * u.x + cs * v.x, sn * u.y + cs * v.y);
-                }
-                double2* ji = Jm + (int64_t)i * ldj;
-                double2* jj = Jm + (int64_t)j * ldj;
-                for (int l = lane; l < r; l += 32) {
-                    const double2 u = ji[l], v = cmul(ph, jj[l]);
-                    ji[l] = make_double2(cs * u.x - sn * v.x, cs * u.y - sn * v.y);
-                    jj[l] = make_double2(sn * u.x + cs * v.x, sn * u.y + cs * v.y);
-                }
+                __syncthreads();
             }
-            __syncthreads();
+            if (tm.size > 1) tm.sync();
         }
-        const int more = *s_flag;
-        __syncthreads();
+        tm.sync();
+        const int more = *(volatile int*)(flag + (sweep & 1));
         if (!more) return sweep + 1;
     }
     return maxsweep + 1;
@@ -285,18 +382,20 @@ __device__ int cta_jacobi(double2* X, int ldx, int rows, int r, double2* Jm, int
 //   the skeleton count is known, j >= it, and the largest remaining column
 //   norm is <= rcond * (largest initial norm).
 // kfix > 0: skeleton count kfix; else the first j with max norm <= eps * max0.
-__device__ void cta_cpqr(double2* A, int ld, int rows, int cols, int extra, int* perm,
+// The outputs are written by CTA 0 and visible to the team on return; ctl: a
+// flag of the team in global memory.
+__device__ void cta_cpqr(const Team& tm, double2* A, int ld, int rows, int cols, int extra, int* perm,
                          double2* diag, double* nrm2, double2* s_v, int kfix, double eps,
-                         double rcond, Red& red, int* out_rank, int* out_k, double* out_eps) {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    for (int c = threadIdx.x; c < cols; c += blockDim.x) perm[c] = c;
-    for (int c = w; c < cols; c += nwarps()) {
+                         double rcond, Red& red, int* out_rank, int* out_k, double* out_eps, int* ctl) {
+    const int lane = threadIdx.x & 31;
+    for (int64_t c = tm.thread(); c < cols; c += tm.threads()) perm[c] = (int)c;
+    for (int c = tm.warp(); c < cols; c += tm.warps()) {
         double s = 0.0;
         for (int i = lane; i < rows; i += 32) s += cabs2(A[(int64_t)c * ld + i]);
         s = warp_sum(s);
         if (lane == 0) nrm2[c] = s;
     }
-    __syncthreads();
+    tm.sync();
     double m0 = 0.0;
     for (int c = threadIdx.x; c < cols; c += blockDim.x) m0 = fmax(m0, nrm2[c]);
     const double max0 = block_max(m0, red);
@@ -305,66 +404,72 @@ __device__ void cta_cpqr(double2* A, int ld, int rows, int cols, int extra, int*
     double eps_ach = 0.0;
     int j = 0;
     for (; j < kmax; ++j) {
-        double mloc = 0.0;
-        for (int c = j + threadIdx.x; c < cols; c += blockDim.x) mloc = fmax(mloc, nrm2[c]);
-        const double mx = block_max(mloc, red);
+        // CTA 0 picks the pivot and brings it to column j
+        if (tm.rank == 0) {
+            double mloc = 0.0;
+            for (int c = j + threadIdx.x; c < cols; c += blockDim.x) mloc = fmax(mloc, nrm2[c]);
+            const double mx = block_max(mloc, red);
+            if (kskel < 0) {
+                if (kfix > 0 && j == kfix) {
+                    kskel = j;
+                    eps_ach = sqrt(mx / max0);
+                } else if (kfix <= 0 && mx <= eps * eps * max0) {
+                    kskel = j;
+                    eps_ach = sqrt(mx / max0);
+                }
+            }
+            const bool stop = (kskel >= 0 && j >= kskel && mx <= rcond * rcond * max0) || mx <= 0.0;
+            if (!stop) {
+                // pivot: lowest original index among the columns within TIE of the max
+                const double thr = (1.0 - TIE) * (1.0 - TIE) * mx;
+                int key = INT_MAX, idx = INT_MAX;
+                for (int c = j + threadIdx.x; c < cols; c += blockDim.x)
+                    if (nrm2[c] >= thr && perm[c] < key) {
+                        key = perm[c];
+                        idx = c;
+                    }
+                const int q = block_argmin(key, idx, red);
+                if (q != j) {
+                    for (int i = threadIdx.x; i < rows; i += blockDim.x) {
+                        const double2 t = A[(int64_t)j * ld + i];
+                        A[(int64_t)j * ld + i] = A[(int64_t)q * ld + i];
+                        A[(int64_t)q * ld + i] = t;
+                    }
+                    __syncthreads();
+                    if (threadIdx.x == 0) {
+                        const int tp = perm[j];
+                        perm[j] = perm[q];
+                        perm[q] = tp;
+                        const double tn = nrm2[j];
+                        nrm2[j] = nrm2[q];
+                        nrm2[q] = tn;
+                    }
+                }
+            }
+            if (threadIdx.x == 0) *(volatile int*)ctl = stop ? 1 : 0;
+        }
+        tm.sync();
+        if (*(volatile int*)ctl) break;
+        householder_step(tm, A, ld, rows, j, cols, cols + extra, diag, nrm2, s_v, red);
+    }
+    if (tm.rank == 0 && threadIdx.x == 0) {
         if (kskel < 0) {
-            if (kfix > 0 && j == kfix) {
-                kskel = j;
-                eps_ach = sqrt(mx / max0);
-            } else if (kfix <= 0 && mx <= eps * eps * max0) {
-                kskel = j;
-                eps_ach = sqrt(mx / max0);
-            }
+            kskel = (kfix > 0) ? min(kfix, j) : j;
+            eps_ach = 0.0;
         }
-        if (kskel >= 0 && j >= kskel && mx <= rcond * rcond * max0) break;
-        if (mx <= 0.0) break;
-        // pivot: lowest original index among the columns within TIE of the max
-        const double thr = (1.0 - TIE) * (1.0 - TIE) * mx;
-        int key = INT_MAX, idx = INT_MAX;
-        for (int c = j + threadIdx.x; c < cols; c += blockDim.x)
-            if (nrm2[c] >= thr && perm[c] < key) {
-                key = perm[c];
-                idx = c;
-            }
-        const int q = block_argmin(key, idx, red);
-        if (q != j) {
-            for (int i = threadIdx.x; i < rows; i += blockDim.x) {
-                const double2 t = A[(int64_t)j * ld + i];
-                A[(int64_t)j * ld + i] = A[(int64_t)q * ld + i];
-                A[(int64_t)q * ld + i] = t;
-            }
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                const int tp = perm[j];
-                perm[j] = perm[q];
-                perm[q] = tp;
-                const double tn = nrm2[j];
-                nrm2[j] = nrm2[q];
-                nrm2[q] = tn;
-            }
-        }
-        __syncthreads();
-        householder_step(A, ld, rows, j, cols, cols + extra, diag, nrm2, s_v, red);
-    }
-    if (kskel < 0) {
-        kskel = (kfix > 0) ? min(kfix, j) : j;
-        eps_ach = 0.0;
-    }
-    if (threadIdx.x == 0) {
         *out_rank = j;
         *out_k = kskel;
         *out_eps = eps_ach;
     }
-    __syncthreads();
+    tm.sync();
 }
 
 // X(0:n, c) = R(0:n, 0:n)^{-1} Bm(0:n, c) for c < ncols, R upper triangular stored
 // above the diagonal of Rm (leading dimension ldr) with its diagonal in diag.
 // One thread per right-hand-side column.  X may alias Bm.
-__device__ void cta_backsub(const double2* Rm, int ldr, const double2* diag, int n,
+__device__ void cta_backsub(const Team& tm, const double2* Rm, int ldr, const double2* diag, int n,
                             const double2* Bm, int ldb, int ncols, double2* X, int ldx) {
-    for (int c = threadIdx.x; c < ncols; c += blockDim.x) {
+    for (int64_t c = tm.thread(); c < ncols; c += tm.threads()) {
         for (int i = n - 1; i >= 0; --i) {
             double2 s = Bm[(int64_t)c * ldb + i];
             for (int l = i + 1; l < n; ++l)
@@ -374,7 +479,7 @@ __device__ void cta_backsub(const double2* Rm, int ldr, const double2* diag, int
             X[(int64_t)c * ldx + i] = cscale(cmulc(d, s), id);  // s / d
         }
     }
-    __syncthreads();
+    tm.sync();
 }
 
 }  // namespace
@@ -411,42 +516,40 @@ __device__ __forceinline__ double2 sketch_entry(int i, int l, unsigned seed, int
 }
 
 template <int DIM>
-__device__ __forceinline__ void sbuild_phase1(SBuildJob& J, double kappa, double rcond, Red& red, double2* s_v) {
-    fill_kernel_matrix<DIM>(J.BD, J.p, J.z, J.p, J.x, J.m, kappa);
-    fill_kernel_matrix<DIM>(J.BD + (int64_t)J.m * J.p, J.p, J.z, J.p, J.y, J.n, kappa);
-    fill_kernel_matrix<DIM>(J.AU, J.m, J.x, J.m, J.y, J.n, kappa);
-    __syncthreads();
+__device__ __forceinline__ void sbuild_phase1(const Team& tm, SBuildJob& J, double kappa, double rcond, Red& red,
+                                              double2* s_v) {
+    fill_kernel_matrix<DIM>(tm, J.BD, J.p, J.z, J.p, J.x, J.m, kappa);
+    fill_kernel_matrix<DIM>(tm, J.BD + (int64_t)J.m * J.p, J.p, J.z, J.p, J.y, J.n, kappa);
+    fill_kernel_matrix<DIM>(tm, J.AU, J.m, J.x, J.m, J.y, J.n, kappa);
+    tm.sync();
     if (J.sketch_d > 0) {
         const int d = J.sketch_d, p = J.p, m = J.m;
-        for (int64_t e = threadIdx.x; e < (int64_t)d * p; e += blockDim.x)
+        for (int64_t e = tm.thread(); e < (int64_t)d * p; e += tm.threads())
             J.OM[e] = sketch_entry((int)(e % d), (int)(e / d), J.seed, J.shape_index);
-        __syncthreads();
-        for (int64_t e = threadIdx.x; e < (int64_t)d * m; e += blockDim.x) {
+        tm.sync();
+        for (int64_t e = tm.thread(); e < (int64_t)d * m; e += tm.threads()) {
             const int i = (int)(e % d), j = (int)(e / d);
             double2 sum = make_double2(0.0, 0.0);
             for (int l = 0; l < p; ++l) sum = cfma(J.OM[(int64_t)l * d + i], J.BD[(int64_t)j * p + l], sum);
             J.Y[e] = sum;
         }
-        __syncthreads();
+        tm.sync();
         // the ID from the sketch: halted at k (a cutoff above every column norm)
-        int rankY;
-        cta_cpqr(J.Y, d, d, m, 0, J.permY, J.diagY, J.nrm2, s_v, J.kfix, 0.0, 2.0, red, &rankY, &J.k,
-                 &J.eps_ach);
+        cta_cpqr(tm, J.Y, d, d, m, 0, J.permY, J.diagY, J.nrm2, s_v, J.kfix, 0.0, 2.0, red, &J.rankB, &J.k,
+                 &J.eps_ach, J.ctl);
         // B's own factorisation, for the least-squares solve of C
-        int kd;
-        double ed;
-        cta_cpqr(J.BD, J.p, J.p, J.m, J.n, J.permB, J.diagB, J.nrm2, s_v, J.kfix, J.eps, B_QR_CUT * rcond, red,
-                 &J.rankB, &kd, &ed);
+        cta_cpqr(tm, J.BD, J.p, J.p, J.m, J.n, J.permB, J.diagB, J.nrm2, s_v, J.kfix, J.eps, B_QR_CUT * rcond, red,
+                 &J.rankB, J.ctl + 1, (double*)(J.ctl + 2), J.ctl);
         return;
     }
-    cta_cpqr(J.BD, J.p, J.p, J.m, J.n, J.permB, J.diagB, J.nrm2, s_v, J.kfix, J.eps, B_QR_CUT * rcond, red,
-             &J.rankB, &J.k, &J.eps_ach);
+    cta_cpqr(tm, J.BD, J.p, J.p, J.m, J.n, J.permB, J.diagB, J.nrm2, s_v, J.kfix, J.eps, B_QR_CUT * rcond, red,
+             &J.rankB, &J.k, &J.eps_ach, J.ctl);
 }
 
 // ----------------------------------------------------------------------------
 // phase 2: Z*, C (minimum norm), U, pivoted QR of A (with U)
 // ----------------------------------------------------------------------------
-__device__ __forceinline__ void sbuild_phase2(SBuildJob& J, double rcond, Red& red, double2* s_v) {
+__device__ __forceinline__ void sbuild_phase2(const Team& tm, SBuildJob& J, double rcond, Red& red, double2* s_v) {
     const int m = J.m, n = J.n, p = J.p, k = J.k, rB = J.rankB;
     // the ID's factorisation: B's own pivoted QR, or the sketch's
     const bool sk = J.sketch_d > 0;
@@ -455,15 +558,15 @@ __device__ __forceinline__ void sbuild_phase2(SBuildJob& J, double rcond, Red& r
     const int* permI = sk ? J.permY : J.permB;
     const double2* diagI = sk ? J.diagY : J.diagB;
     // skeleton indices
-    for (int i = threadIdx.x; i < k; i += blockDim.x) J.skel[i] = permI[i];
+    for (int64_t i = tm.thread(); i < k; i += tm.threads()) J.skel[i] = permI[i];
     // Z* (k x m, ld k): identity on the skeleton, T = R11^{-1} R12 elsewhere
-    for (int64_t e = threadIdx.x; e < (int64_t)k * m; e += blockDim.x) J.Zs[e] = make_double2(0.0, 0.0);
-    __syncthreads();
-    for (int i = threadIdx.x; i < k; i += blockDim.x)
+    for (int64_t e = tm.thread(); e < (int64_t)k * m; e += tm.threads()) J.Zs[e] = make_double2(0.0, 0.0);
+    tm.sync();
+    for (int64_t i = tm.thread(); i < k; i += tm.threads())
         J.Zs[(int64_t)permI[i] * k + i] = make_double2(1.0, 0.0);
     // T columns: solve into the work area W1 (k x (m-k), ld k)
-    cta_backsub(RI, ldi, diagI, k, RI + (int64_t)k * ldi, ldi, m - k, J.W1, k);
-    for (int64_t e = threadIdx.x; e < (int64_t)k * (m - k); e += blockDim.x) {
+    cta_backsub(tm, RI, ldi, diagI, k, RI + (int64_t)k * ldi, ldi, m - k, J.W1, k);
+    for (int64_t e = tm.thread(); e < (int64_t)k * (m - k); e += tm.threads()) {
         const int i = (int)(e % k), c = (int)(e / k);
         J.Zs[(int64_t)permI[k + c] * k + i] = J.W1[e];
     }
@@ -479,7 +582,7 @@ __device__ __forceinline__ void sbuild_phase2(SBuildJob& J, double rcond, Red& r
     {
         const int L = m - rB + 1;
         double2* V = J.XB;
-        const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = nwarps();
+        const int lane = threadIdx.x & 31;
         // entry l of row r's reduced vector: column r (l = 0) or column rB + l - 1
         auto col_of = [&](int r, int l) { return l == 0 ? r : rB + l - 1; };
         if (L > 1) {
@@ -505,78 +608,85 @@ __device__ __forceinline__ void sbuild_phase2(SBuildJob& J, double rcond, Red& r
                     } else {
                         const double2 u = J.BD[(int64_t)col_of(i, l) * p + i];
                         v = cscale(make_double2(u.x, -u.y), inv);
-                        J.BD[(int64_t)col_of(i, l) * p + i] = make_double2(0.0, 0.0);
                     }
-                    V[(int64_t)i * L + l] = v;
+                    s_v[l] = v;
                 }
-                __syncthreads();  // every thread has read R(i, i) before it is replaced
-                if (threadIdx.x == 0) J.diagB[i] = make_double2(alpha.x, -alpha.y);
+                __syncthreads();
                 // rows r < i: w <- w P_i = w - 2 (w . v) v^H
-                for (int r = w; r < i; r += nw) {
+                for (int r = tm.warp(); r < i; r += tm.warps()) {
                     double2 d = make_double2(0.0, 0.0);
-                    for (int l = lane; l < L; l += 32)
-                        d = cfma(J.BD[(int64_t)col_of(i, l) * p + r], V[(int64_t)i * L + l], d);
+                    for (int l = lane; l < L; l += 32) d = cfma(J.BD[(int64_t)col_of(i, l) * p + r], s_v[l], d);
                     d = cscale(warp_sum2(d), 2.0);
                     for (int l = lane; l < L; l += 32) {
                         double2& x = J.BD[(int64_t)col_of(i, l) * p + r];
-                        x = cfmsc(V[(int64_t)i * L + l], d, x);  // x - conj(v_l) d
+                        x = cfmsc(s_v[l], d, x);  // x - conj(v_l) d
                     }
+                }
+                tm.sync();  // every CTA has read row i and R(i, i)
+                if (tm.rank == 0) {
+                    for (int l = threadIdx.x; l < L; l += blockDim.x) {
+                        V[(int64_t)i * L + l] = s_v[l];
+                        if (l > 0) J.BD[(int64_t)col_of(i, l) * p + i] = make_double2(0.0, 0.0);
+                    }
+                    if (threadIdx.x == 0) J.diagB[i] = make_double2(alpha.x, -alpha.y);
                 }
                 __syncthreads();
             }
+            tm.sync();
         }
         // Y = T^{-1} (Q_B^H D)(0:rB, :) into W2 (rB x n, ld rB), T now in R_B's place
         const int ldy = rB > 0 ? rB : 1;
-        cta_backsub(J.BD, p, J.diagB, rB, J.BD + (int64_t)m * p, p, n, J.W2, ldy);
-        for (int64_t e = threadIdx.x; e < (int64_t)m * n; e += blockDim.x) {
+        cta_backsub(tm, J.BD, p, J.diagB, rB, J.BD + (int64_t)m * p, p, n, J.W2, ldy);
+        for (int64_t e = tm.thread(); e < (int64_t)m * n; e += tm.threads()) {
             const int i = (int)(e % m), c = (int)(e / m);
             J.W3[e] = i < rB ? J.W2[(int64_t)c * ldy + i] : make_double2(0.0, 0.0);
         }
-        __syncthreads();
-        // W3 <- P_{rB-1} ... P_0 W3 (P_0 first), P_i x = x - 2 v (v^H x)
+        tm.sync();
+        // W3 <- P_{rB-1} ... P_0 W3 (P_0 first), P_i x = x - 2 v (v^H x); a column
+        // stays with one warp
         if (L > 1) {
-            for (int i = 0; i < rB; ++i) {
-                for (int c = w; c < n; c += nw) {
+            for (int c = tm.warp(); c < n; c += tm.warps()) {
+                for (int i = 0; i < rB; ++i) {
                     double2* x = J.W3 + (int64_t)c * m;
                     double2 d = make_double2(0.0, 0.0);
                     for (int l = lane; l < L; l += 32) d = cfmac(V[(int64_t)i * L + l], x[col_of(i, l)], d);
                     d = cscale(warp_sum2(d), 2.0);
                     for (int l = lane; l < L; l += 32)
                         x[col_of(i, l)] = cfms(V[(int64_t)i * L + l], d, x[col_of(i, l)]);
+                    __syncwarp();  // x[i] is read by another lane in a later step
                 }
-                __syncthreads();
             }
+            tm.sync();
         }
     }
-    for (int64_t e = threadIdx.x; e < (int64_t)m * n; e += blockDim.x) {
+    for (int64_t e = tm.thread(); e < (int64_t)m * n; e += tm.threads()) {
         const int i = (int)(e % m), c = (int)(e / m);
         J.C[(int64_t)c * m + J.permB[i]] = J.W3[e];
     }
     // U = (Z*)^T into AU columns n..n+k-1 (m x k, ld m)
-    __syncthreads();
-    for (int64_t e = threadIdx.x; e < (int64_t)m * k; e += blockDim.x) {
+    tm.sync();
+    for (int64_t e = tm.thread(); e < (int64_t)m * k; e += tm.threads()) {
         const int i = (int)(e % m), c = (int)(e / m);
         J.AU[(int64_t)(n + c) * m + i] = J.Zs[(int64_t)i * k + c];
     }
-    __syncthreads();
+    tm.sync();
     // pivoted QR of A (m x n), reflectors applied to U, run down to the
     // rounding level: the truncation itself is done on the singular values
     const double rq = 0.01 * rcond;
-    int kdummy;
-    double edummy;
-    cta_cpqr(J.AU, m, m, n, k, J.permA, J.diagA, J.nrm2, s_v, -1, rq, rq, red, &J.rankA, &kdummy,
-             &edummy);
+    cta_cpqr(tm, J.AU, m, m, n, k, J.permA, J.diagA, J.nrm2, s_v, -1, rq, rq, red, &J.rankA, J.ctl + 1,
+             (double*)(J.ctl + 2), J.ctl);
 }
 
 // ----------------------------------------------------------------------------
 // phase 3: truncated SVD of A from its pivoted QR (one-sided Jacobi on
 // R_A^H), the factors of A^+, and S
 // ----------------------------------------------------------------------------
-__device__ __forceinline__ void sbuild_phase3(SBuildJob& J, double rcond, Red& red, int& s_flag, int& s_r) {
+__device__ __forceinline__ void sbuild_phase3(const Team& tm, SBuildJob& J, double rcond, Red& red, int& s_r,
+                                              JacobiShared& jac) {
     const int m = J.m, n = J.n, k = J.k, rA = J.rankA;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31;
     // X = R_A^H (n x rA, ld n) and J = I (rA x rA, ld n)
-    for (int64_t e = threadIdx.x; e < (int64_t)n * rA; e += blockDim.x) {
+    for (int64_t e = tm.thread(); e < (int64_t)n * rA; e += tm.threads()) {
         const int c = (int)(e % n), i = (int)(e / n);
         double2 v = make_double2(0.0, 0.0);
         if (c == i)
@@ -585,21 +695,21 @@ __device__ __forceinline__ void sbuild_phase3(SBuildJob& J, double rcond, Red& r
             v = J.AU[(int64_t)c * m + i];
         J.XA[e] = make_double2(v.x, -v.y);
     }
-    for (int64_t e = threadIdx.x; e < (int64_t)rA * rA; e += blockDim.x) {
+    for (int64_t e = tm.thread(); e < (int64_t)rA * rA; e += tm.threads()) {
         const int l = (int)(e % rA), i = (int)(e / rA);
         J.JA[(int64_t)i * n + l] = make_double2(l == i ? 1.0 : 0.0, 0.0);
     }
-    __syncthreads();
+    tm.sync();
     const double tol = 2.220446049250313e-16 * sqrt((double)max(n, 1));
-    const int sweeps = cta_jacobi(J.XA, n, n, rA, J.JA, n, tol, 60, &s_flag);
+    const int sweeps = cta_jacobi(tm, J.XA, n, n, rA, J.JA, n, tol, 60, J.ctl, jac);
     // singular values = column norms of X J
-    for (int i = w; i < rA; i += nwarps()) {
+    for (int i = tm.warp(); i < rA; i += tm.warps()) {
         double sum = 0.0;
         for (int l = lane; l < n; l += 32) sum = abs2_acc(J.XA[(int64_t)i * n + l], sum);
         sum = warp_sum(sum);
         if (lane == 0) J.sig[i] = sqrt(sum);
     }
-    __syncthreads();
+    tm.sync();
     double mloc = 0.0;
     for (int i = threadIdx.x; i < rA; i += blockDim.x) mloc = fmax(mloc, J.sig[i]);
     const double smax = block_max(mloc, red);
@@ -608,14 +718,16 @@ __device__ __forceinline__ void sbuild_phase3(SBuildJob& J, double rcond, Red& r
         for (int i = 0; i < rA; ++i)
             if (J.sig[i] > rcond * smax) J.keep[r++] = i;
         s_r = r;
-        J.rankS = r;
-        J.sweepsA = sweeps;
+        if (tm.rank == 0) {
+            J.rankS = r;
+            J.sweepsA = sweeps;
+        }
     }
     __syncthreads();
     const int r = s_r;
     // F = P_A V_r Sigma_r^{-1} = P_A (X J)(:, kept) Sigma_r^{-2}  (n x r, ld n, rows in
     // the original column order of A)
-    for (int64_t e = threadIdx.x; e < (int64_t)n * r; e += blockDim.x) {
+    for (int64_t e = tm.thread(); e < (int64_t)n * r; e += tm.threads()) {
         const int row = (int)(e % n), slot = (int)(e / n);
         const int i = J.keep[slot];
         const double sg = J.sig[i];
@@ -623,15 +735,16 @@ __device__ __forceinline__ void sbuild_phase3(SBuildJob& J, double rcond, Red& r
     }
     // kept columns of J moved to the front, in order (a source column is never
     // the destination of an earlier one)
-    for (int slot = 0; slot < r; ++slot) {
+    for (int slot = 0; tm.rank == 0 && slot < r; ++slot) {
         const int i = J.keep[slot];
         if (i != slot)
             for (int l = threadIdx.x; l < rA; l += blockDim.x)
                 J.JA[(int64_t)slot * n + l] = J.JA[(int64_t)i * n + l];
         __syncthreads();
     }
+    tm.sync();
     // M = Z* C (k x n, ld k) into W1
-    for (int64_t e = threadIdx.x; e < (int64_t)k * n; e += blockDim.x) {
+    for (int64_t e = tm.thread(); e < (int64_t)k * n; e += tm.threads()) {
         const int i = (int)(e % k), c = (int)(e / k);
         double2 sum = make_double2(0.0, 0.0);
         for (int l = 0; l < m; ++l) sum = cfma(J.Zs[(int64_t)l * k + i], J.C[(int64_t)c * m + l], sum);
@@ -639,31 +752,33 @@ __device__ __forceinline__ void sbuild_phase3(SBuildJob& J, double rcond, Red& r
     }
     // H = J_r^H (Q_A^H U)(0:rA, :)  (r x k, ld r) into W3
     const int ldh = r > 0 ? r : 1;
-    for (int64_t e = threadIdx.x; e < (int64_t)r * k; e += blockDim.x) {
+    for (int64_t e = tm.thread(); e < (int64_t)r * k; e += tm.threads()) {
         const int i = (int)(e % ldh), c = (int)(e / ldh);
         double2 sum = make_double2(0.0, 0.0);
         for (int l = 0; l < rA; ++l)
             sum = cfmac(J.JA[(int64_t)i * n + l], J.AU[(int64_t)(n + c) * m + l], sum);
         J.W3[e] = sum;
     }
-    __syncthreads();
+    tm.sync();
     // G = M F  (k x r, ld k) into XB
-    for (int64_t e = threadIdx.x; e < (int64_t)k * r; e += blockDim.x) {
+    for (int64_t e = tm.thread(); e < (int64_t)k * r; e += tm.threads()) {
         const int i = (int)(e % k), c = (int)(e / k);
         double2 sum = make_double2(0.0, 0.0);
         for (int l = 0; l < n; ++l) sum = cfma(J.W1[(int64_t)l * k + i], J.FA[(int64_t)c * n + l], sum);
         J.XB[e] = sum;
     }
-    __syncthreads();
+    tm.sync();
     // S = G H  (k x k, ld k), and its Frobenius norm
-    double sq = 0.0;
-    for (int64_t e = threadIdx.x; e < (int64_t)k * k; e += blockDim.x) {
+    for (int64_t e = tm.thread(); e < (int64_t)k * k; e += tm.threads()) {
         const int i = (int)(e % k), c = (int)(e / k);
         double2 sum = make_double2(0.0, 0.0);
         for (int l = 0; l < r; ++l) sum = cfma(J.XB[(int64_t)l * k + i], J.W3[(int64_t)c * ldh + l], sum);
         J.S[e] = sum;
-        sq += cabs2(sum);
     }
+    tm.sync();
+    if (tm.rank != 0) return;
+    double sq = 0.0;
+    for (int64_t e = threadIdx.x; e < (int64_t)k * k; e += blockDim.x) sq += cabs2(J.S[e]);
     sq = block_sum(sq, red);
     if (threadIdx.x == 0) J.snorm = sqrt(sq);
 }
@@ -683,31 +798,45 @@ __device__ __forceinline__ int next_job(int* counter, int* s_job) {
     return j;
 }
 
+// f(team, job) for the jobs of this CTA, or the one job of the cluster of `size`
+// CTAs that it belongs to.  One call site: two copies of a phase may contract
+// their products and sums differently.
+template <typename F>
+__device__ __forceinline__ void each_job(int size, int njobs, int* counter, int* s_job, F&& f) {
+    const Team tm{size > 1 ? (int)(blockIdx.x % size) : 0, size};
+    int j = size > 1 ? (int)(blockIdx.x / size) : next_job(counter, s_job);
+    while (j < njobs) {
+        f(tm, j);
+        j = size > 1 ? njobs : next_job(counter, s_job);
+    }
+}
+
 template <int DIM>
-__global__ void __launch_bounds__(SBT_MAX) sbuild_phase1_kernel(SBuildJob* jobs, int njobs, int* counter,
+__global__ void __launch_bounds__(SBT_MAX) sbuild_phase1_kernel(SBuildJob* jobs, int njobs, int* counter, int team,
                                                                 double kappa, double rcond) {
     __shared__ Red red;
     __shared__ int s_job;
     extern __shared__ double2 s_v[];
-    for (int j = next_job(counter, &s_job); j < njobs; j = next_job(counter, &s_job))
-        sbuild_phase1<DIM>(jobs[j], kappa, rcond, red, s_v);
+    each_job(team, njobs, counter, &s_job,
+             [&](const Team& tm, int j) { sbuild_phase1<DIM>(tm, jobs[j], kappa, rcond, red, s_v); });
 }
 
-__global__ void __launch_bounds__(SBT_MAX) sbuild_phase2_kernel(SBuildJob* jobs, int njobs, int* counter,
+__global__ void __launch_bounds__(SBT_MAX) sbuild_phase2_kernel(SBuildJob* jobs, int njobs, int* counter, int team,
                                                                 double rcond) {
     __shared__ Red red;
     __shared__ int s_job;
     extern __shared__ double2 s_v[];
-    for (int j = next_job(counter, &s_job); j < njobs; j = next_job(counter, &s_job))
-        sbuild_phase2(jobs[j], rcond, red, s_v);
+    each_job(team, njobs, counter, &s_job,
+             [&](const Team& tm, int j) { sbuild_phase2(tm, jobs[j], rcond, red, s_v); });
 }
 
-__global__ void __launch_bounds__(SBT_MAX) sbuild_phase3_kernel(SBuildJob* jobs, int njobs, int* counter,
+__global__ void __launch_bounds__(SBT_MAX) sbuild_phase3_kernel(SBuildJob* jobs, int njobs, int* counter, int team,
                                                                 double rcond) {
     __shared__ Red red;
-    __shared__ int s_job, s_flag, s_r;
-    for (int j = next_job(counter, &s_job); j < njobs; j = next_job(counter, &s_job))
-        sbuild_phase3(jobs[j], rcond, red, s_flag, s_r);
+    __shared__ int s_job, s_r;
+    __shared__ JacobiShared jac;
+    each_job(team, njobs, counter, &s_job,
+             [&](const Team& tm, int j) { sbuild_phase3(tm, jobs[j], rcond, red, s_r, jac); });
 }
 
 // ----------------------------------------------------------------------------
@@ -1013,12 +1142,32 @@ __global__ void __launch_bounds__(32 * RB) recon_block_kernel(const RhsBody* __r
 }
 
 template <typename K>
-static int blocks_per_sm(K kern, int threads, size_t sm) {
+static int blocks_per_sm(K* kern, int threads, size_t sm) {
     if (sm > 48 * 1024)
         MBS_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
     int nb = 0;
     MBS_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, threads, sm));
     return std::max(nb, 1);
+}
+
+// Launch of a build phase: a persistent grid of single CTAs, or one cluster of
+// `team` CTAs per job.
+template <typename... A>
+static void launch_phase(void (*kern)(A...), int njobs, int team, int threads, size_t sm, cudaStream_t st, A... args) {
+    const int per = blocks_per_sm(kern, threads, sm);
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)(team > 1 ? njobs * team : std::min(njobs, mbs_num_sms() * per)));
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = sm;
+    cfg.stream = st;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = (unsigned)team;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = team > 1 ? 1 : 0;
+    MBS_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, args...));
+    MBS_CHECK_LAUNCH();
 }
 
 void launch_sbuild(int dim, SBuildJob* d_jobs, int njobs, int* d_counter, int rows_max, int threads,
@@ -1027,22 +1176,20 @@ void launch_sbuild(int dim, SBuildJob* d_jobs, int njobs, int* d_counter, int ro
     if (threads != 128 && threads != 256 && threads != 512)
         throw MbsError{MBS_ERR_ARG, "S build: threads per CTA must be 128, 256 or 512"};
     const size_t sm = (size_t)std::max(rows_max, 1) * sizeof(double2);
-    const int nsm = mbs_num_sms();
+    // CTAs per shape: a shape alone on an SM is bound by that SM's FP64 pipe and
+    // by the latency of its steps, so few shapes are shared out over clusters of
+    // up to 8 CTAs (the portable size) while every CTA still finds an SM.  Phases
+    // 1, 2 and 3 of 3 shapes with 128 points: 8.7, 5.9, 28.1 ms to 2.6, 3.2,
+    // 6.3 ms; of 6 ellipsoids with 192: 17.2, 9.2, 15.7 ms to 4.5, 5.4, 4.3 ms.
+    int team = 8;
+    while (team > 1 && njobs * team > mbs_num_sms()) team /= 2;
     MBS_CUDA_TRY(cudaMemsetAsync(d_counter, 0, 3 * sizeof(int), st));
-    if (dim == 2) {
-        const int g = std::min(njobs, nsm * blocks_per_sm(sbuild_phase1_kernel<2>, threads, sm));
-        sbuild_phase1_kernel<2><<<g, threads, sm, st>>>(d_jobs, njobs, d_counter, kappa, rcond);
-    } else {
-        const int g = std::min(njobs, nsm * blocks_per_sm(sbuild_phase1_kernel<3>, threads, sm));
-        sbuild_phase1_kernel<3><<<g, threads, sm, st>>>(d_jobs, njobs, d_counter, kappa, rcond);
-    }
-    MBS_CHECK_LAUNCH();
-    int g = std::min(njobs, nsm * blocks_per_sm(sbuild_phase2_kernel, threads, sm));
-    sbuild_phase2_kernel<<<g, threads, sm, st>>>(d_jobs, njobs, d_counter + 1, rcond);
-    MBS_CHECK_LAUNCH();
-    g = std::min(njobs, nsm * blocks_per_sm(sbuild_phase3_kernel, threads, 0));
-    sbuild_phase3_kernel<<<g, threads, 0, st>>>(d_jobs, njobs, d_counter + 2, rcond);
-    MBS_CHECK_LAUNCH();
+    if (dim == 2)
+        launch_phase(sbuild_phase1_kernel<2>, njobs, team, threads, sm, st, d_jobs, njobs, d_counter, team, kappa, rcond);
+    else
+        launch_phase(sbuild_phase1_kernel<3>, njobs, team, threads, sm, st, d_jobs, njobs, d_counter, team, kappa, rcond);
+    launch_phase(sbuild_phase2_kernel, njobs, team, threads, sm, st, d_jobs, njobs, d_counter + 1, team, rcond);
+    launch_phase(sbuild_phase3_kernel, njobs, team, threads, (size_t)0, st, d_jobs, njobs, d_counter + 2, team, rcond);
 }
 
 void launch_rhs(const RhsBody* d_bodies, int T, int nrhs, int mmax, int nmax, const double2* v,

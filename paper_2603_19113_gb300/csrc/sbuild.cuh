@@ -34,6 +34,7 @@ struct SBuildJob {
     int* permB;     // m
     double2* diagB; // min(p, m)
     int* permA;     // n
+    int* ctl;       // 4: the factorisations' flags and unused outputs
     double2* diagA; // n
     double2* JA;    // n x n (kept): accumulated rotations, kept columns first
     double2* FA;    // n x n (kept): F = P_A V_r Sigma_r^{-1}, first rankS columns
