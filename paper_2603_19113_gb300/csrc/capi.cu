@@ -1584,81 +1584,107 @@ void build(mbs_ctx* c, int nshapes, const mbs_shape* shapes, int nbodies, const 
         }
         const int nj = (int)batch.size();
         std::vector<SBuildJob> jobs(nj);
-        std::vector<void*> tmp;
-        auto talloc = [&](size_t bytes) {
-            void* p = dalloc(c, bytes);
-            tmp.push_back(p);
-            return p;
-        };
-        int pmax = 1, mmax = 1;
-        for (int j = 0; j < nj; ++j) {
-            ShapeHost& s = c->shapes[batch[j]];
-            SBuildJob& J = jobs[j];
-            std::memset(&J, 0, sizeof(J));
-            const int kcap = s.kfix > 0 ? s.kfix : std::min(s.m, s.p);
-            J.m = s.m;
-            J.n = s.n;
-            J.p = s.p;
-            J.kfix = s.kfix;
-            J.eps = s.eps;
-            const int dsk = s.kfix + c->opt.id_sketch;
-            J.sketch_d = (c->opt.id_sketch > 0 && s.kfix > 0 && dsk < s.p) ? dsk : 0;
-            J.seed = c->opt.id_seed;
-            J.shape_index = batch[j];
-            if (J.sketch_d > 0) {
-                J.OM = (double2*)talloc(sizeof(double2) * (size_t)J.sketch_d * s.p);
-                J.Y = (double2*)talloc(sizeof(double2) * (size_t)J.sketch_d * s.m);
-                J.permY = (int*)talloc(sizeof(int) * s.m);
-                J.diagY = (double2*)talloc(sizeof(double2) * std::min(J.sketch_d, s.m));
+        // One allocation for the batch's work arrays, one for what is kept, one
+        // upload of the point sets and one readback of the skeletons: allocating
+        // and copying them one by one took a quarter of the build of 300 2D
+        // shapes (about 100 of 400 ms).
+        struct Slab {
+            char* base = nullptr;
+            size_t used = 0;
+            void* take(size_t bytes) {
+                void* p = base ? base + used : nullptr;
+                used += (bytes + 127) & ~(size_t)127;
+                return p;
             }
-            s.dx = galloc<double>(c, s.x.size());
-            s.dy = galloc<double>(c, s.y.size());
-            s.dz = galloc<double>(c, s.z.size());
-            MBS_CUDA_TRY(cudaMemcpyAsync(s.dx, s.x.data(), s.x.size() * 8, cudaMemcpyHostToDevice, c->st));
-            MBS_CUDA_TRY(cudaMemcpyAsync(s.dy, s.y.data(), s.y.size() * 8, cudaMemcpyHostToDevice, c->st));
-            MBS_CUDA_TRY(cudaMemcpyAsync(s.dz, s.z.data(), s.z.size() * 8, cudaMemcpyHostToDevice, c->st));
-            J.x = s.dx;
-            J.y = s.dy;
-            J.z = s.dz;
-            J.BD = (double2*)talloc(sizeof(double2) * (size_t)s.p * (s.m + s.n));
-            s.AU = galloc<double2>(c, (size_t)s.m * (s.n + kcap));
-            J.AU = s.AU;
-            J.W1 = (double2*)talloc(sizeof(double2) * (size_t)kcap * std::max(s.m, s.n));
-            J.W2 = (double2*)talloc(sizeof(double2) * (size_t)std::min(s.p, s.m) * s.n);
-            J.W3 = (double2*)talloc(sizeof(double2) * (size_t)s.m * s.n);
-            J.XB = (double2*)talloc(sizeof(double2) * (size_t)s.m * std::min(s.p, s.m));
-            J.XA = (double2*)talloc(sizeof(double2) * (size_t)s.n * s.n);
-            J.sig = (double*)talloc(sizeof(double) * s.n);
-            J.keep = (int*)talloc(sizeof(int) * s.n);
-            J.nrm2 = (double*)talloc(sizeof(double) * std::max(s.m, s.n));
-            J.permB = (int*)talloc(sizeof(int) * s.m);
-            J.diagB = (double2*)talloc(sizeof(double2) * std::min(s.p, s.m));
-            J.permA = (int*)talloc(sizeof(int) * s.n);
-            J.ctl = (int*)talloc(sizeof(int) * 4);
-            J.diagA = (double2*)talloc(sizeof(double2) * s.n);
-            s.JA = galloc<double2>(c, (size_t)s.n * s.n);
-            s.FA = galloc<double2>(c, (size_t)s.n * s.n);
-            J.JA = s.JA;
-            J.FA = s.FA;
-            J.skel = (int*)talloc(sizeof(int) * kcap);
-            s.Zs = galloc<double2>(c, (size_t)kcap * s.m);
-            s.C = galloc<double2>(c, (size_t)s.m * s.n);
-            s.S64 = galloc<double2>(c, (size_t)kcap * kcap);
-            J.Zs = s.Zs;
-            J.C = s.C;
-            J.S = s.S64;
-            pmax = std::max(pmax, s.p);
-            mmax = std::max(mmax, s.m);
+        } tmp, keep, pts, skels;
+        int pmax = 1, mmax = 1;
+        auto assign = [&]() {
+            tmp.used = keep.used = pts.used = skels.used = 0;
+            for (int j = 0; j < nj; ++j) {
+                ShapeHost& s = c->shapes[batch[j]];
+                SBuildJob& J = jobs[j];
+                std::memset(&J, 0, sizeof(J));
+                const int kcap = s.kfix > 0 ? s.kfix : std::min(s.m, s.p);
+                J.m = s.m;
+                J.n = s.n;
+                J.p = s.p;
+                J.kfix = s.kfix;
+                J.eps = s.eps;
+                const int dsk = s.kfix + c->opt.id_sketch;
+                J.sketch_d = (c->opt.id_sketch > 0 && s.kfix > 0 && dsk < s.p) ? dsk : 0;
+                J.seed = c->opt.id_seed;
+                J.shape_index = batch[j];
+                auto t2 = [&](size_t count) { return (double2*)tmp.take(sizeof(double2) * count); };
+                auto k2 = [&](size_t count) { return (double2*)keep.take(sizeof(double2) * count); };
+                auto ti = [&](size_t count) { return (int*)tmp.take(sizeof(int) * count); };
+                if (J.sketch_d > 0) {
+                    J.OM = t2((size_t)J.sketch_d * s.p);
+                    J.Y = t2((size_t)J.sketch_d * s.m);
+                    J.permY = ti(s.m);
+                    J.diagY = t2(std::min(J.sketch_d, s.m));
+                }
+                J.x = s.dx = (double*)pts.take(s.x.size() * 8);
+                J.y = s.dy = (double*)pts.take(s.y.size() * 8);
+                J.z = s.dz = (double*)pts.take(s.z.size() * 8);
+                J.BD = t2((size_t)s.p * (s.m + s.n));
+                J.AU = s.AU = k2((size_t)s.m * (s.n + kcap));
+                J.W1 = t2((size_t)kcap * std::max(s.m, s.n));
+                J.W2 = t2((size_t)std::min(s.p, s.m) * s.n);
+                J.W3 = t2((size_t)s.m * s.n);
+                J.XB = t2((size_t)s.m * std::min(s.p, s.m));
+                J.XA = t2((size_t)s.n * s.n);
+                J.sig = (double*)tmp.take(sizeof(double) * s.n);
+                J.keep = ti(s.n);
+                J.nrm2 = (double*)tmp.take(sizeof(double) * std::max(s.m, s.n));
+                J.permB = ti(s.m);
+                J.diagB = t2(std::min(s.p, s.m));
+                J.permA = ti(s.n);
+                J.ctl = ti(4);
+                J.diagA = t2(s.n);
+                J.JA = s.JA = k2((size_t)s.n * s.n);
+                J.FA = s.FA = k2((size_t)s.n * s.n);
+                J.skel = (int*)skels.take(sizeof(int) * kcap);
+                J.Zs = s.Zs = k2((size_t)kcap * s.m);
+                J.C = s.C = k2((size_t)s.m * s.n);
+                J.S = s.S64 = k2((size_t)kcap * kcap);
+                pmax = std::max(pmax, s.p);
+                mmax = std::max(mmax, s.m);
+            }
+        };
+        assign();  // sizes
+        const size_t tmp_bytes = tmp.used, skel_bytes = skels.used;
+        std::vector<char> hpts(pts.used), hskel(skel_bytes);
+        keep.base = (char*)galloc<char>(c, keep.used);
+        pts.base = (char*)galloc<char>(c, pts.used);
+        tmp.base = (char*)dalloc(c, tmp_bytes + skel_bytes + sizeof(SBuildJob) * nj + 256);
+        struct Freed {  // also when the build fails
+            mbs_ctx* c;
+            void* p;
+            ~Freed() {
+                cudaStreamSynchronize(c->st);
+                dfree(c, p);
+            }
+        } freed{c, tmp.base};
+        skels.base = tmp.base + tmp_bytes;
+        assign();  // addresses
+        for (int j = 0; j < nj; ++j) {
+            const ShapeHost& s = c->shapes[batch[j]];
+            std::memcpy(hpts.data() + ((char*)s.dx - pts.base), s.x.data(), s.x.size() * 8);
+            std::memcpy(hpts.data() + ((char*)s.dy - pts.base), s.y.data(), s.y.size() * 8);
+            std::memcpy(hpts.data() + ((char*)s.dz - pts.base), s.z.data(), s.z.size() * 8);
         }
-        SBuildJob* d_jobs = (SBuildJob*)talloc(sizeof(SBuildJob) * nj);
-        int* d_counter = (int*)talloc(3 * sizeof(int));
+        MBS_CUDA_TRY(cudaMemcpyAsync(pts.base, hpts.data(), hpts.size(), cudaMemcpyHostToDevice, c->st));
+        SBuildJob* d_jobs = (SBuildJob*)(skels.base + skel_bytes);
+        int* d_counter = (int*)(((uintptr_t)(d_jobs + nj) + 127) & ~(uintptr_t)127);
         MBS_CUDA_TRY(cudaMemcpyAsync(d_jobs, jobs.data(), sizeof(SBuildJob) * nj, cudaMemcpyHostToDevice, c->st));
         const int rows_max = std::max(pmax, mmax);
         const int threads = sbuild_threads(c, d_jobs, nj, d_counter, rows_max);
         launch_sbuild(d, d_jobs, nj, d_counter, rows_max, threads, c->kappa, c->opt.ls_rcond, c->st);
         c->last_sbuild_threads = threads;
         MBS_CUDA_TRY(cudaMemcpyAsync(jobs.data(), d_jobs, sizeof(SBuildJob) * nj, cudaMemcpyDeviceToHost, c->st));
+        MBS_CUDA_TRY(cudaMemcpyAsync(hskel.data(), skels.base, skel_bytes, cudaMemcpyDeviceToHost, c->st));
         MBS_CUDA_TRY(cudaStreamSynchronize(c->st));
+        size_t s32 = 0;
         for (int j = 0; j < nj; ++j) {
             ShapeHost& s = c->shapes[batch[j]];
             const SBuildJob& J = jobs[j];
@@ -1670,14 +1696,18 @@ void build(mbs_ctx* c, int nshapes, const mbs_shape* shapes, int nbodies, const 
             s.snorm = J.snorm;
             s.eps_ach = J.eps_ach;
             if (s.k < 1) throw MbsError{MBS_ERR_ARG, "shape " + std::to_string(batch[j]) + ": zero skeleton"};
-            s.skel.resize(s.k);
-            MBS_CUDA_TRY(cudaMemcpy(s.skel.data(), J.skel, s.k * sizeof(int), cudaMemcpyDeviceToHost));
-            // Z* and S were written with leading dimension k (<= kcap): already compact.
-            s.S32 = galloc<float2>(c, (size_t)s.k * s.k);
+            const int* sk = (const int*)(hskel.data() + ((char*)J.skel - skels.base));
+            s.skel.assign(sk, sk + s.k);
+            s32 += (size_t)s.k * s.k;
+        }
+        // Z* and S were written with leading dimension k (<= kcap): already compact.
+        float2* S32 = galloc<float2>(c, s32);
+        for (int j = 0; j < nj; ++j) {
+            ShapeHost& s = c->shapes[batch[j]];
+            s.S32 = S32;
+            S32 += (size_t)s.k * s.k;
             launch_f64_to_f32(s.S64, s.S32, (int64_t)s.k * s.k, c->st);
         }
-        MBS_CUDA_TRY(cudaStreamSynchronize(c->st));
-        for (void* p : tmp) dfree(c, p);
     }
     setup_layout(c);
     c->built = true;
