@@ -1240,58 +1240,26 @@ mbs_status guarded(mbs_ctx* c, F&& f) {
     }
 }
 
-// For every target (SoA dim x M, host or device), the body whose proxy
-// surface strictly contains it, or -1; proxies are disjoint, so there is at
-// most one.  A hash grid of cell size = the largest proxy radius finds the
-// candidate bodies.  Throws MBS_ERR_ARG on a non-finite target.
-std::vector<int> proxy_bodies(mbs_ctx* c, const double* pts, int64_t M);
-
 bool finite_all(const double* p, size_t n) {
     for (size_t i = 0; i < n; ++i)
         if (!std::isfinite(p[i])) return false;
     return true;
 }
 
-std::vector<int> proxy_bodies(mbs_ctx* c, const double* pts, int64_t M) {
-    const int d = c->dim;
-    std::vector<double> hp((size_t)d * M);
-    if (is_device_ptr(pts))
-        MBS_CUDA_TRY(cudaMemcpy(hp.data(), pts, hp.size() * sizeof(double), cudaMemcpyDeviceToHost));
-    else
-        std::memcpy(hp.data(), pts, hp.size() * sizeof(double));
-    if (!finite_all(hp.data(), hp.size())) throw MbsError{MBS_ERR_ARG, "non-finite target"};
+// For every target (device, SoA dim x M), the body whose proxy surface strictly
+// contains it, or -1, into d_tb; returns the first target inside a proxy (-1:
+// none).  Throws MBS_ERR_ARG on a non-finite target.
+int64_t proxy_bodies(mbs_ctx* c, const double* d_pts, int64_t M, int* d_tb) {
     double reach = 0;
     for (int t = 0; t < c->T; ++t) reach = std::max(reach, c->shapes[c->bodies[t].shape].proxy_radius);
-    const double h = std::max(reach, 1e-12);
-    std::unordered_map<int64_t, std::vector<int>> grid;
-    auto key = [&](int64_t ix, int64_t iy, int64_t iz) {
-        return ((ix & 0x1FFFFF) << 42) | ((iy & 0x1FFFFF) << 21) | (iz & 0x1FFFFF);
-    };
-    for (int t = 0; t < c->T; ++t) {
-        const double* cc = c->bodies[t].c;
-        grid[key((int64_t)std::floor(cc[0] / h), (int64_t)std::floor(cc[1] / h),
-                 d == 3 ? (int64_t)std::floor(cc[2] / h) : 0)]
-            .push_back(t);
-    }
-    std::vector<int> tb((size_t)M, -1);
-    for (int64_t i = 0; i < M; ++i) {
-        double p3[3] = {hp[i], hp[(size_t)M + i], d == 3 ? hp[(size_t)2 * M + i] : 0.0};
-        const int64_t ix = (int64_t)std::floor(p3[0] / h), iy = (int64_t)std::floor(p3[1] / h),
-                      iz = d == 3 ? (int64_t)std::floor(p3[2] / h) : 0;
-        for (int64_t a = -1; a <= 1; ++a)
-            for (int64_t b2 = -1; b2 <= 1; ++b2)
-                for (int64_t e = (d == 3 ? -1 : 0); e <= (d == 3 ? 1 : 0); ++e) {
-                    auto it = grid.find(key(ix + a, iy + b2, iz + e));
-                    if (it == grid.end()) continue;
-                    for (int t : it->second) {
-                        const double pr = c->shapes[c->bodies[t].shape].proxy_radius;
-                        double r2 = 0;
-                        for (int q = 0; q < d; ++q) r2 += (p3[q] - c->bodies[t].c[q]) * (p3[q] - c->bodies[t].c[q]);
-                        if (r2 < pr * pr * (1.0 - 1e-12)) tb[i] = t;
-                    }
-                }
-    }
-    return tb;
+    long long* d_first = scratch<long long>(c, "near_first", 2);  // first near target, first non-finite one
+    launch_proxy_bodies(c->dim, M, d_pts, c->T, c->d_centres, c->d_centres + (size_t)4 * c->T, std::max(reach, 1e-12),
+                        d_tb, d_first, c->st);
+    long long first[2];
+    MBS_CUDA_TRY(cudaMemcpyAsync(first, d_first, sizeof(first), cudaMemcpyDeviceToHost, c->st));
+    MBS_CUDA_TRY(cudaStreamSynchronize(c->st));
+    if (first[1] < M) throw MbsError{MBS_ERR_ARG, "non-finite target"};
+    return first[0] < M ? first[0] : -1;
 }
 
 void world_point(const mbs_body& B, int dim, const double* loc, double* out) {
@@ -1386,13 +1354,14 @@ void setup_layout(mbs_ctx* c) {
     std::vector<int> body(N);
     std::vector<float> loc32((size_t)d * N);
     c->skel_world.assign((size_t)d * N, 0.0);
-    // centres (3 per body) followed by the bounding radius of every body
-    std::vector<double> cen((size_t)4 * T, 0.0);
+    // centres (3 per body) followed by the bounding and the proxy radius of every body
+    std::vector<double> cen((size_t)5 * T, 0.0);
     for (int t = 0; t < T; ++t) {
         const mbs_body& B = c->bodies[t];
         const ShapeHost& s = c->shapes[B.shape];
         for (int a = 0; a < 3; ++a) cen[3 * t + a] = (a < d) ? B.c[a] : 0.0;
         cen[(size_t)3 * T + t] = s.bound_radius;
+        cen[(size_t)4 * T + t] = s.proxy_radius;
         for (int i = 0; i < s.k; ++i) {
             const int64_t g = c->off[t] + i;
             body[g] = t;
@@ -1409,7 +1378,7 @@ void setup_layout(mbs_ctx* c) {
     c->d_off = galloc<int64_t>(c, T + 1);
     c->d_loc32 = galloc<float>(c, (size_t)d * N);
     c->d_xw64 = galloc<double>(c, (size_t)d * N);
-    c->d_centres = galloc<double>(c, (size_t)4 * T);
+    c->d_centres = galloc<double>(c, (size_t)5 * T);
     c->d_pair = galloc<float4>(c, (size_t)T * T);
     c->d_pair_phi0 = d == 3 ? galloc<float>(c, (size_t)T * T) : nullptr;
     MBS_CUDA_TRY(cudaMemcpyAsync(c->d_body, body.data(), N * sizeof(int), cudaMemcpyHostToDevice, c->st));
@@ -2118,13 +2087,16 @@ mbs_status mbs_evaluate_field(mbs_ctx* c, int nrhs, int64_t M, const double* pts
             throw MbsError{MBS_ERR_ARG, "bad sizes or null pointer"};
         if (M == 0) return MBS_OK;
         // targets must lie on or outside every proxy surface
-        const std::vector<int> tb = proxy_bodies(c, pts, M);
-        for (int64_t i = 0; i < M; ++i)
-            if (tb[i] >= 0)
-                throw MbsError{MBS_ERR_NEAR_TARGET, "target " + std::to_string(i) +
-                                                        " lies inside the proxy surface of body " +
-                                                        std::to_string(tb[i])};
         const double* dp = in_dev_real(c, pts, (size_t)c->dim * M, "io_pts");
+        // into the partial sums' buffer, which the evaluation below overwrites
+        int* d_tb = reinterpret_cast<int*>(scratch<double2>(c, "part_field", (size_t)M * nrhs));
+        const int64_t i = proxy_bodies(c, dp, M, d_tb);
+        if (i >= 0) {
+            int tb = -1;
+            MBS_CUDA_TRY(cudaMemcpy(&tb, d_tb + i, sizeof(int), cudaMemcpyDeviceToHost));
+            throw MbsError{MBS_ERR_NEAR_TARGET, "target " + std::to_string(i) +
+                                                    " lies inside the proxy surface of body " + std::to_string(tb)};
+        }
         const double2* dq = in_dev(c, qhat, (size_t)c->N * nrhs, "io_q");
         OutBuf ou = out_dev(c, u, (size_t)M * nrhs, "io_u");
         field64(c, nrhs, M, dp, dq, ou.dev, nullptr);
@@ -2159,10 +2131,9 @@ mbs_status mbs_evaluate_field_near(mbs_ctx* c, int nrhs, int64_t M, const double
         if (nrhs < 1 || M < 0 || (M > 0 && (!pts || !qhat || !qmfs || !u)))
             throw MbsError{MBS_ERR_ARG, "bad sizes or null pointer"};
         if (M == 0) return MBS_OK;
-        const std::vector<int> tb = proxy_bodies(c, pts, M);
-        int* d_tb = scratch<int>(c, "near_tb", (size_t)M);
-        MBS_CUDA_TRY(cudaMemcpyAsync(d_tb, tb.data(), (size_t)M * sizeof(int), cudaMemcpyHostToDevice, c->st));
         const double* dp = in_dev_real(c, pts, (size_t)c->dim * M, "io_pts");
+        int* d_tb = scratch<int>(c, "near_tb", (size_t)M);
+        proxy_bodies(c, dp, M, d_tb);
         const double2* dq = in_dev(c, qhat, (size_t)c->N * nrhs, "io_q");
         const double2* dm = in_dev(c, qmfs, (size_t)c->Nm * nrhs, "io_qmfs_in");
         OutBuf ou = out_dev(c, u, (size_t)M * nrhs, "io_u");

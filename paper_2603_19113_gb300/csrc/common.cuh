@@ -147,6 +147,13 @@ void launch_field_f64(const GLayout& L, double kappa, int64_t M, const double* t
                       const double2* q, double2* u, double2* part, int nsplit,
                       const int* d_split_body, cudaStream_t st, const int* tbody = nullptr);
 
+// tb[i] = the body whose proxy surface strictly contains target i, or -1;
+// first[0], first[1]: the smallest index of a target inside a proxy and of a
+// non-finite one (M or more: none).  centres [T][3], prox [T], cell >= every
+// proxy radius.
+void launch_proxy_bodies(int dim, int64_t M, const double* pts, int T, const double* centres, const double* prox,
+                         double cell, int* tb, long long* first, cudaStream_t st);
+
 // MFS sources of one placed body (Sec. 4.6 reconstruction): y_world = c + R y_local.
 struct MfsBody {
     const double* y;  // local MFS sources, SoA dim x n (the shape's device copy)

@@ -533,6 +533,68 @@ void launch_f64_dim(int64_t Nt, const double* tgt, const int* tbody, int64_t Ns,
     }
 }
 
+// Which proxy holds a target.  One thread per target against all bodies, staged
+// through shared memory as floats: a pair is looked at in FP64 only where the
+// FP32 distance, less its rounding, is below the proxy radius.  A hash grid on
+// the host, rebuilt for every call, with a copy of the targets there, took 0.65
+// ms of a field call on 4096 targets and 1000 bodies (6.68 ms to 6.03 ms) and
+// 0.76 ms on 3001 and 40 in 3D (1.83 ms to 1.07 ms).  Of several bodies the one
+// that a walk over the neighbouring grid cells, x slowest, meets last is taken.
+constexpr int PB = 128;
+template <int DIM>
+__global__ void __launch_bounds__(PB) proxy_bodies_kernel(const int64_t M, const double* __restrict__ pts, const int T,
+                                                          const double* __restrict__ centres,
+                                                          const double* __restrict__ prox, const double cell,
+                                                          int* __restrict__ tb, long long* __restrict__ first) {
+    __shared__ float4 s_b[PB];
+    const int64_t i = (int64_t)blockIdx.x * PB + threadIdx.x;
+    double x[3] = {0.0, 0.0, 0.0};
+    bool fine = true;
+    if (i < M)
+#pragma unroll
+        for (int a = 0; a < DIM; ++a) {
+            x[a] = pts[a * M + i];
+            fine = fine && isfinite(x[a]);
+        }
+    const float xf = (float)x[0], yf = (float)x[1], zf = (float)x[2];
+    const float reach = 1e-6f * (fabsf(xf) + fabsf(yf) + fabsf(zf));
+    long long best = -1;
+    for (int t0 = 0; t0 < T; t0 += PB) {
+        __syncthreads();
+        const int t = t0 + threadIdx.x;
+        if (t < T) {
+            const double* c = centres + 3 * (int64_t)t;
+            const float p = (float)prox[t];
+            s_b[threadIdx.x] = make_float4((float)c[0], (float)c[1], (float)c[2],
+                                           p * 1.00001f + 1e-6f * (float)(fabs(c[0]) + fabs(c[1]) + fabs(c[2])));
+        }
+        __syncthreads();
+        const int n = min(PB, T - t0);
+        for (int k = 0; k < n; ++k) {
+            const float4 b = s_b[k];
+            const float dx = xf - b.x, dy = yf - b.y, dz = DIM == 3 ? zf - b.z : 0.f, lim = b.w + reach;
+            if (!(fmaf(dx, dx, fmaf(dy, dy, dz * dz)) > lim * lim)) {  // also where FP32 overflows
+                const double* c = centres + 3 * (int64_t)(t0 + k);
+                double r2 = 0.0;
+#pragma unroll
+                for (int a = 0; a < DIM; ++a) r2 += (x[a] - c[a]) * (x[a] - c[a]);
+                const double pr = prox[t0 + k];
+                if (r2 < pr * pr * (1.0 - 1e-12)) {
+                    long long where = 0;
+#pragma unroll
+                    for (int a = 0; a < 3; ++a)
+                        where = 3 * where + (a < DIM ? (long long)(floor(c[a] / cell) - floor(x[a] / cell)) + 1 : 1);
+                    best = max(best, where * T + (t0 + k));
+                }
+            }
+        }
+    }
+    if (i >= M) return;
+    tb[i] = best < 0 ? -1 : (int)(best % T);
+    if (best >= 0) atomicMin(first, (long long)i);
+    if (!fine) atomicMin(first + 1, (long long)i);
+}
+
 // Sec. 4.6: the field of body tau at a target inside its proxy surface from its
 // reconstructed MFS sources, added to u.  One thread per (target, RHS).
 template <int DIM>
@@ -648,6 +710,17 @@ void launch_field_f64(const GLayout& L, double kappa, int64_t M, const double* t
                           d_split_body, st);
     const int64_t len = M * nrhs;
     reduce_splits_kernel<double2><<<(unsigned)((len + 255) / 256), 256, 0, st>>>(part, nsplit, len, u);
+    MBS_CHECK_LAUNCH();
+}
+
+void launch_proxy_bodies(int dim, int64_t M, const double* pts, int T, const double* centres, const double* prox,
+                         double cell, int* tb, long long* first, cudaStream_t st) {
+    MBS_CUDA_TRY(cudaMemsetAsync(first, 0x7f, 2 * sizeof(long long), st));
+    const unsigned g = (unsigned)((M + PB - 1) / PB);
+    if (dim == 2)
+        proxy_bodies_kernel<2><<<g, PB, 0, st>>>(M, pts, T, centres, prox, cell, tb, first);
+    else
+        proxy_bodies_kernel<3><<<g, PB, 0, st>>>(M, pts, T, centres, prox, cell, tb, first);
     MBS_CHECK_LAUNCH();
 }
 
