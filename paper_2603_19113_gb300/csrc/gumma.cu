@@ -27,8 +27,8 @@
 //   - A and D are single-buffered in tensor memory: a phi warp evaluates the
 //     first half of the next chunk, then waits for the previous chunk's MMAs
 //     before it overwrites A; D accumulates one source body (a "segment") at a
-//     time, and when a body ends every thread adds its row of D into FP32
-//     registers before it signals the next chunk, whose first MMA resets D,
+//     time, and when a body ends every thread adds its row of D into its FP32
+//     sums before it signals the next chunk, whose first MMA resets D,
 //     so the tensor-core accumulation never runs over more than one body.
 // Every wait is bounded (about 2 s): on a timeout the kernel sets *err, writes
 // NaN to its outputs, waits (bounded) for its work in flight, frees its tensor
@@ -62,6 +62,7 @@ struct UmmaCfg {
     static constexpr uint32_t LBO = (NM / 8) * 128;    // K-direction core-matrix stride
     static constexpr uint32_t SBO = 128;               // N-direction core-matrix stride
     // kind::tf32, D f32, A/B tf32, both K-major, N = NM, M = 128
+    static_assert(UM_STAGES * REC + UM_T * NM * 4 <= UM_SMEM, "ring and sums");
     static constexpr uint32_t IDESC = (1u << 4) | (2u << 7) | (2u << 10) |
                                       ((uint32_t)(NM >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
 };
@@ -185,7 +186,9 @@ __global__ void __launch_bounds__(128) g_umma_pack_kernel(const GLayout L, const
 // 2D: VF selects the x >= 64 fit of H0 (degree 2) for body pairs whose points
 // are all that far apart, else the x >= 8 fit (degree 4) (modulus fits with
 // the amplitude constant folded in, in K); glast is the last phase
-// coefficient plus the body-pair phase.
+// coefficient plus the body-pair phase.  Which products are fused into the sums
+// behind them is written out: left to the compiler it changes with the code
+// around it, and the result with it (by 1e-6, the rounding of phases near 100).
 template <int DIM, bool VF>
 __device__ __forceinline__ float2 far_pair(const float4 sj, const float A0, const float Bx,
                                            const float By, const float Bz, const float R,
@@ -196,10 +199,10 @@ __device__ __forceinline__ float2 far_pair(const float4 sj, const float A0, cons
         const float* gc = VF ? c_f32_64G : c_f32_8G;
         const float* fcoef = VF ? K.f64a : K.f8a;
         const float s = fmaf(Bx, sj.x, fmaf(By, sj.y, A0 + sj.w));
-        const float r2 = R2 + s;
+        const float r2 = fmaf(R, R, s);
         const float rinv = rsqrtf(r2);
-        const float r = r2 * rinv;
-        const float dr = __fdividef(s, r + R);
+        const float r = __fmul_rn(r2, rinv);
+        const float dr = __fdividef(s, __fadd_rn(r, R));
         const float u = fmaf(VF ? K.c64 : K.c8, rinv, -1.f);
         float f = fcoef[0], gp = gc[0];
 #pragma unroll
@@ -210,8 +213,8 @@ __device__ __forceinline__ float2 far_pair(const float4 sj, const float A0, cons
         f = fmaf(f, u, fcoef[DEG]);
         gp = fmaf(gp, u, glast);
         const float2 e = expi_f32(fmaf(K.kappa, dr, gp));
-        const float amp = f * rsqrtf(r);
-        return make_float2(amp * e.x, amp * e.y);
+        const float amp = __fmul_rn(f, rsqrtf(r));
+        return make_float2(__fmul_rn(amp, e.x), __fmul_rn(amp, e.y));
     } else {
         const float s = fmaf(Bx, sj.x, fmaf(By, sj.y, fmaf(Bz, sj.z, A0 + sj.w)));
         const float r2 = R2 + s;
@@ -372,9 +375,11 @@ __global__ void __launch_bounds__(UM_THREADS, 4) g_umma_kernel(const GLayout L, 
         const uint32_t a_lane = tmem + ((uint32_t)(warp * 32) << 16);
 
 
-        float accr[NR], acci[NR];
+        // the sums over the bodies so far: needed once a body, so they sit in shared
+        // memory, [column / 4][target] (in registers, the 16-RHS kernel spilled)
+        float4* acc = reinterpret_cast<float4*>(um_smem + UM_STAGES * C::REC) + tid;
 #pragma unroll
-        for (int r = 0; r < NR; ++r) accr[r] = acci[r] = 0.f;
+        for (int k = 0; k < C::NM / 4; ++k) acc[k * UM_T] = make_float4(0.f, 0.f, 0.f, 0.f);
         auto read_d = [&]() {
             uint32_t v[16];
 #pragma unroll
@@ -382,12 +387,13 @@ __global__ void __launch_bounds__(UM_THREADS, 4) g_umma_kernel(const GLayout L, 
                 tmem_ld16(a_lane + 64 + 16 * h, v);
                 asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-                for (int e = 0; e < 16; ++e) {
-                    const int col = 16 * h + e;
-                    if (col < NR)
-                        accr[col] += __uint_as_float(v[e]);
-                    else
-                        acci[col - NR] += __uint_as_float(v[e]);
+                for (int e = 0; e < 4; ++e) {
+                    float4 x = acc[(4 * h + e) * UM_T];
+                    x.x += __uint_as_float(v[4 * e]);
+                    x.y += __uint_as_float(v[4 * e + 1]);
+                    x.z += __uint_as_float(v[4 * e + 2]);
+                    x.w += __uint_as_float(v[4 * e + 3]);
+                    acc[(4 * h + e) * UM_T] = x;
                 }
             }
         };
@@ -535,9 +541,15 @@ __global__ void __launch_bounds__(UM_THREADS, 4) g_umma_kernel(const GLayout L, 
         if (valid) {
             const float nanv = __int_as_float(0x7fc00000);
 #pragma unroll
-            for (int r = 0; r < NR; ++r)
-                if (r0 + r < nrhs)
-                    out[(int64_t)(r0 + r) * N + i] = abort ? make_float2(nanv, nanv) : make_float2(accr[r], acci[r]);
+            for (int k = 0; k < NR / 4; ++k) {
+                const float4 re = acc[k * UM_T], im = acc[(NR / 4 + k) * UM_T];
+                const float2 y[4] = {make_float2(re.x, im.x), make_float2(re.y, im.y), make_float2(re.z, im.z),
+                                     make_float2(re.w, im.w)};
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    if (r0 + 4 * k + e < nrhs)
+                        out[(int64_t)(r0 + 4 * k + e) * N + i] = abort ? make_float2(nanv, nanv) : y[e];
+            }
         }
     }
     tc_fence_before();
