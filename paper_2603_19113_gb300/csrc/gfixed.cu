@@ -8,7 +8,7 @@
 // the right-hand sides, integers of 60 bits relative to the largest |q| of a
 // source body, takes 4 wide multiply-adds and 8 FP32 ones (the cross terms of
 // high and low words, whose 24 bits end near 2^-56) a pair and right-hand side,
-// and goes into FP64 sums once per round of 64 sources.
+// and goes into FP64 sums once per 64 sources.
 //
 // g_fx_pack_kernel, one CTA per body, turns the offsets from the body's centre
 // and the right-hand sides into integers scaled by the body's own radius and
@@ -16,6 +16,8 @@
 // 1e-270..1e270, is marked and its sums are formed in FP64 from the caller's
 // values; so are bodies outside the formats of phi_fx.h (targets close to the
 // hull of a body, extreme kappa or sizes) and 2D pairs below kappa r = 4.
+#include <type_traits>
+
 #include "bessel.cuh"
 #include "common.cuh"
 #include "fx_tables.h"
@@ -26,7 +28,8 @@ namespace {
 __device__ const FxSteps g_fx_steps = fx_steps();
 
 constexpr int FXT = 128;     // threads per CTA
-constexpr int FX_SB = 64;    // sources staged per round
+constexpr int FX_SB = 32;    // sources staged per round
+constexpr int FX_FLUSH = 64; // sources per integer sum
 constexpr int FX_QBITS = 60;  // right-hand sides are integers below 2^60: 64 products stay below 2^62 in an integer sum
 constexpr int FX_CROSS = 4;   // sources per FP32 sum of cross terms (below 2^63: its integer part fits 32 bits)
 constexpr int FX_BAD = INT_MIN;  // stored exponent of a body whose values need FP64
@@ -107,7 +110,7 @@ __device__ __noinline__ double2 fx_phi_f64(double kappa, double r2) {
 // staged sources of the same targets (small problems, where the sources of a
 // body would otherwise be one long chain per thread).
 template <int DIM, int NR, int SG>
-__global__ void __launch_bounds__(FXT, 4)
+__global__ void __launch_bounds__(FXT, 5)
     g_fx_kernel(const FxKappa kap, const int64_t Nt, const double* __restrict__ tgt, const int* __restrict__ tbody,
                 const int64_t N, const int T, const double* __restrict__ xw, const int64_t* __restrict__ off,
                 const double* __restrict__ centres, const FxPacked P, const int nrhs, const int r0,
@@ -160,7 +163,6 @@ __global__ void __launch_bounds__(FXT, 4)
             }
         };
         auto flush = [&]() {
-            carry();
 #pragma unroll
             for (int r = 0; r < NR; ++r)
                 if (r0 + r < nrhs) {
@@ -172,6 +174,7 @@ __global__ void __launch_bounds__(FXT, 4)
                     ar[r] = ai[r] = 0;
                 }
         };
+        int since = 0;
         for (int64_t jc = js; jc < je; jc += FX_SB) {
             const int n = (int)min((int64_t)FX_SB, je - jc);
             __syncthreads();
@@ -216,7 +219,12 @@ __global__ void __launch_bounds__(FXT, 4)
                     }
                     if ((j - k0) % FX_CROSS == FX_CROSS - 1) carry();
                 }
-                flush();
+                carry();
+                since += FX_SB;
+                if (since == FX_FLUSH || jc + FX_SB >= je) {
+                    flush();
+                    since = 0;
+                }
             } else if (act) {
 #pragma unroll 1
                 for (int j = k0; j < k1; ++j) {
@@ -251,22 +259,21 @@ template <int DIM, int SG>
 void launch_fx(const GLayout& L, const double* centres, const FxKappa& k, int64_t Nt, const double* tgt, const int* tbody,
                int nrhs, const double2* q, const FxPacked& P, double2* part, int nsplit, const int* sb, cudaStream_t st) {
     const dim3 grid((unsigned)((Nt + FXT / SG - 1) / (FXT / SG)), (unsigned)nsplit);
+    auto pass = [&](auto width, int r0) {
+        g_fx_kernel<DIM, decltype(width)::value, SG>
+            <<<grid, FXT, 0, st>>>(k, Nt, tgt, tbody, L.N, L.T, L.xw64, L.off, centres, P, nrhs, r0, q, part, sb);
+        MBS_CHECK_LAUNCH();
+        return r0 + decltype(width)::value;
+    };
+    // a right-hand side of padding costs about 4 % of a pair
     for (int r0 = 0; r0 < nrhs;) {
         const int left = nrhs - r0;
-        if (left > 4) {
-            g_fx_kernel<DIM, 8, SG><<<grid, FXT, 0, st>>>(k, Nt, tgt, tbody, L.N, L.T, L.xw64, L.off, centres, P, nrhs, r0, q, part, sb);
-            r0 += 8;
-        } else if (left > 2) {
-            g_fx_kernel<DIM, 4, SG><<<grid, FXT, 0, st>>>(k, Nt, tgt, tbody, L.N, L.T, L.xw64, L.off, centres, P, nrhs, r0, q, part, sb);
-            r0 += 4;
-        } else if (left == 2) {
-            g_fx_kernel<DIM, 2, SG><<<grid, FXT, 0, st>>>(k, Nt, tgt, tbody, L.N, L.T, L.xw64, L.off, centres, P, nrhs, r0, q, part, sb);
-            r0 += 2;
-        } else {
-            g_fx_kernel<DIM, 1, SG><<<grid, FXT, 0, st>>>(k, Nt, tgt, tbody, L.N, L.T, L.xw64, L.off, centres, P, nrhs, r0, q, part, sb);
-            r0 += 1;
-        }
-        MBS_CHECK_LAUNCH();
+        r0 = left > 6    ? pass(std::integral_constant<int, 8>{}, r0)
+             : left > 4  ? pass(std::integral_constant<int, 6>{}, r0)
+             : left == 4 ? pass(std::integral_constant<int, 4>{}, r0)
+             : left == 3 ? pass(std::integral_constant<int, 3>{}, r0)
+             : left == 2 ? pass(std::integral_constant<int, 2>{}, r0)
+                         : pass(std::integral_constant<int, 1>{}, r0);
     }
 }
 
