@@ -516,7 +516,11 @@ Shape32 shape32(mbs_ctx* c, int nrhs, const float2* x, float2* y) {
     if (c->opt.mac_path == 0 && h.path == 3) paths.push_back(1);
     for (int p : paths) {
         const int base = choose_nsplit(c, p == 3 ? 2 * c->N : c->N);
-        for (int ns : {base, base / 2, 2 * base}) {
+        for (int ns : {base, base / 2, 2 * base, 4 * base}) {
+            // four times the usual count: small CTAs even out bodies of uneven
+            // size (700 bodies, 16 right-hand sides: 4.64 ms with 14 splits, 4.30
+            // with 28); the FP32-pipe kernel gains nothing
+            if (ns == 4 * base && p != 3) continue;
             ns = std::max(1, std::min(ns, max_nsplit(c)));
             bool dup = false;
             for (const Shape32& q : cand) dup = dup || (q.path == p && q.nsplit == ns);
@@ -529,7 +533,12 @@ Shape32 shape32(mbs_ctx* c, int nrhs, const float2* x, float2* y) {
     launch_g32(c, nrhs, x, y, cand[0], nullptr, nullptr);  // warm-up
     for (size_t ci = 0; ci < cand.size(); ++ci) {
         MBS_CUDA_TRY(cudaEventRecord(a, c->st));
-        launch_g32(c, nrhs, x, y, cand[ci], nullptr, nullptr);
+        try {
+            launch_g32(c, nrhs, x, y, cand[ci], nullptr, nullptr);
+        } catch (const MbsError& e) {
+            if (e.st != MBS_ERR_NOMEM || ci == 0) throw;
+            continue;  // no memory for that many partial sums
+        }
         MBS_CUDA_TRY(cudaEventRecord(b, c->st));
         MBS_CUDA_TRY(cudaEventSynchronize(b));
         float ms = 0.f;
@@ -562,15 +571,33 @@ void G32(mbs_ctx* c, int nrhs, const float2* x, float2* y) {
     c->last_path = sh.path;
     c->last_nsplit = sh.nsplit;
 }
-// Source splits of the fixed-point kernel: about four rounds of CTAs.
+// Source splits of the fixed-point kernel: about eight rounds of CTAs (four
+// measured 2 % slower at 237 bodies and 5 right-hand sides).
 int fx_nsplit(mbs_ctx* c, int64_t ntargets) {
-    return choose_nsplit(c, ntargets * 256 / fx_tile(ntargets, c->T));
+    if (c->opt.tile_override > 0) return choose_nsplit(c, ntargets);
+    const int64_t tile = fx_tile(ntargets, c->T), tiles = (ntargets + tile - 1) / tile;
+    const int64_t ns = (32LL * mbs_num_sms() + tiles - 1) / std::max<int64_t>(1, tiles);
+    return (int)std::max<int64_t>(1, std::min<int64_t>(ns, std::min(c->T, 256)));
+}
+
+// Partial sums of the FP64-accurate kernels: for the fixed-point kernel's splits
+// where there is memory for them, at least for the others'.
+double2* part64(mbs_ctx* c, const char* name, int ns64, int nsfx, size_t len) {
+    if (nsfx > ns64) {
+        try {
+            return scratch<double2>(c, name, nsfx * len);
+        } catch (const MbsError& e) {
+            if (e.st != MBS_ERR_NOMEM) throw;
+            c->fx_off = true;
+        }
+    }
+    return scratch<double2>(c, name, ns64 * len);
 }
 
 void G64(mbs_ctx* c, int nrhs, const double2* x, double2* y) {
     const bool want_fx = c->opt.fp64_kernel == 2 && !c->fx_off;
     const int ns64 = choose_nsplit(c, c->N), nsfx = want_fx ? fx_nsplit(c, c->N) : 0;
-    double2* part = scratch<double2>(c, "part64", (size_t)std::max(ns64, nsfx) * nrhs * c->N);
+    double2* part = part64(c, "part64", ns64, nsfx, (size_t)nrhs * c->N);
     int* sb = split_table(c, ns64);
     int* sbfx = want_fx ? split_table(c, nsfx) : nullptr;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -600,7 +627,7 @@ void G64(mbs_ctx* c, int nrhs, const double2* x, double2* y) {
 void field64(mbs_ctx* c, int nrhs, int64_t M, const double* pts, const double2* q, double2* u, const int* tbody) {
     const bool want_fx = c->opt.fp64_kernel == 2 && !c->fx_off;
     const int ns64 = choose_nsplit(c, M), nsfx = want_fx ? fx_nsplit(c, M) : 0;
-    double2* part = scratch<double2>(c, "part_field", (size_t)std::max(ns64, nsfx) * nrhs * M);
+    double2* part = part64(c, "part_field", ns64, nsfx, (size_t)nrhs * M);
     int* sb = split_table(c, ns64);
     int* sbfx = want_fx ? split_table(c, nsfx) : nullptr;
     if (void* pack = fx_workspace(c, nrhs))
