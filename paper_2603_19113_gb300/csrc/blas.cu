@@ -199,27 +199,29 @@ __global__ void __launch_bounds__(256) dots_kernel(const V* __restrict__ basis, 
     }
 }
 
-// out[ir] = sum over blk of partial[ir * nblk + blk]: one warp per output,
-// each lane sums a fixed stride of the partials in order, then an xor tree
-// (every lane ends with the same, reproducible total).
-__global__ void dots_finish_kernel(const double2* __restrict__ partial, int count, int nblk,
-                                   double2* __restrict__ out) {
-    const int ir = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-    const int lane = threadIdx.x & 31;
-    if (ir >= count) return;
-    const double2* __restrict__ p = partial + (int64_t)ir * nblk;
+// out[ir] = sum over blk of partial[ir * nblk + blk]: LP lanes per output, each
+// sums a fixed stride of the partials in order, then an xor tree (every lane
+// ends with the same, reproducible total).  The tree's FP64 additions bind it,
+// so few partials take few lanes (10,800 outputs of 14: 10.4 us with 32 lanes,
+// 6.3 us with 8).
+template <int LP>
+__global__ void __launch_bounds__(256) dots_finish_kernel(const double2* __restrict__ partial, int count, int nblk,
+                                                          double2* __restrict__ out) {
+    const int ir = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / LP);
+    const int lane = threadIdx.x % LP;
+    const double2* __restrict__ p = partial + (int64_t)min(ir, count - 1) * nblk;
     double sx = 0.0, sy = 0.0;
-    for (int b = lane; b < nblk; b += 32) {
+    for (int b = lane; b < nblk; b += LP) {
         const double2 v = p[b];
         sx += v.x;
         sy += v.y;
     }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
+    for (int o = LP / 2; o > 0; o >>= 1) {
         sx += __shfl_xor_sync(0xffffffffu, sx, o);
         sy += __shfl_xor_sync(0xffffffffu, sy, o);
     }
-    if (lane == 0) out[ir] = make_double2(sx, sy);
+    if (lane == 0 && ir < count) out[ir] = make_double2(sx, sy);
 }
 
 // w_r += sign * sum_i basis_{i,r} h[i * nrhs + r]
@@ -374,10 +376,10 @@ __global__ void __launch_bounds__(256) chol_small_kernel(const double2* __restri
             const double d = g[k * s + k].x;
             if (!(d > 1e-13 * s_gmax)) {
                 s_bad = 1;
-            } else {
-                const double r = sqrt(d);
-                g[k * s + k] = make_double2(r, 0.0);
-                s_inv = 1.0 / r;
+            } else {  // one chain of dependent FP64 operations instead of a root and a division
+                const double inv = rsqrt(d);
+                g[k * s + k] = make_double2(d * inv, 0.0);
+                s_inv = inv;
             }
         }
         __syncthreads();
@@ -962,6 +964,13 @@ void launch_sapply_f64(const SBlocks& B, int64_t N, int nrhs, const double2* x, 
     MBS_CHECK_LAUNCH();
 }
 
+static void launch_finish(const double2* partial, int count, int nblk, double2* out, cudaStream_t st) {
+    if (nblk <= 64)
+        dots_finish_kernel<8><<<nblocks((int64_t)count * 8), 256, 0, st>>>(partial, count, nblk, out);
+    else
+        dots_finish_kernel<32><<<nblocks((int64_t)count * 32), 256, 0, st>>>(partial, count, nblk, out);
+}
+
 template <typename V>
 void launch_dots(const V* basis, int nvec, const V* w, int64_t N, int nrhs, double2* out,
                  double2* scratch, int nblk, cudaStream_t st) {
@@ -981,7 +990,7 @@ void launch_dots(const V* basis, int nvec, const V* w, int64_t N, int nrhs, doub
     dots_kernel<V><<<g, 256, sm, st>>>(basis, nvec, w, N, nrhs, nblk == 1 ? out : scratch, nblk, per);
     MBS_CHECK_LAUNCH();
     if (nblk == 1) return;
-    dots_finish_kernel<<<nblocks((int64_t)nvec * nrhs * 32, 256), 256, 0, st>>>(scratch, nvec * nrhs, nblk, out);
+    launch_finish(scratch, nvec * nrhs, nblk, out, st);
     MBS_CHECK_LAUNCH();
 }
 
@@ -989,13 +998,17 @@ template <typename V>
 void launch_update(const V* basis, int nvec, const double2* h, V* w, int64_t N, int nrhs,
                    double sign, cudaStream_t st) {
     if (nvec == 0) return;
-    const unsigned gx = (unsigned)std::min<int64_t>((N + 255) / 256, 4 * mbs_num_sms());
+    // Short vectors take CTAs of one warp: a row costs 4 FP64 multiply-adds a
+    // vector, which bind the few SMs that 256-thread CTAs would leave it to (16 us
+    // for 40 vectors of 640 on three SMs).
+    const int th = N * nrhs < 256LL * mbs_num_sms() ? 32 : 256;
+    const unsigned gx = (unsigned)std::min<int64_t>((N + th - 1) / th, 4 * mbs_num_sms());
     dim3 g(gx, (unsigned)nrhs);
     const size_t sm = (size_t)nvec * sizeof(V);
     if (sm > 48 * 1024)
         MBS_CUDA_TRY(cudaFuncSetAttribute(update_kernel<V>,
                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    update_kernel<V><<<g, 256, sm, st>>>(basis, nvec, h, w, N, nrhs, sign);
+    update_kernel<V><<<g, th, sm, st>>>(basis, nvec, h, w, N, nrhs, sign);
     MBS_CHECK_LAUNCH();
 }
 
@@ -1171,7 +1184,7 @@ void launch_ts_gram(const V* A, int ka, const V* B, int kb, int64_t N, double2* 
         ts_gram_kernel<V><<<g, 256, 0, st>>>(A, ka, B, kb, N, scratch, nblk);
     }
     MBS_CHECK_LAUNCH();
-    dots_finish_kernel<<<nblocks((int64_t)ka * kb * 32, 256), 256, 0, st>>>(scratch, ka * kb, nblk, C);
+    launch_finish(scratch, ka * kb, nblk, C, st);
     MBS_CHECK_LAUNCH();
 }
 
