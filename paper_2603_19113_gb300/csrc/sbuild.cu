@@ -950,7 +950,7 @@ __global__ void __launch_bounds__(256) recon_kernel(const RhsBody* __restrict__ 
 
 // ----------------------------------------------------------------------------
 // The same for bodies of at most 256 collocation points: one CTA per body and
-// block of 8 right-hand sides, one warp per right-hand side through the
+// block of up to 8 right-hand sides (rhs_per_cta), one warp per right-hand side through the
 // reflectors, then all threads over the entries of the five products.
 //
 // The FP64 pipe bounds this (64 cycles a warp instruction and scheduler).  The
@@ -1080,16 +1080,16 @@ __device__ __forceinline__ void block_Apinv(const RhsBody& B, double2* t, double
 }
 
 __global__ void __launch_bounds__(32 * RB) rhs_block_kernel(const RhsBody* __restrict__ bodies, const int nrhs,
-                                                            const int mmax, const int nmax,
+                                                            const int rb, const int mmax, const int nmax,
                                                             const double2* __restrict__ v, const int64_t Mtot,
                                                             double2* __restrict__ b, const int64_t N) {
     extern __shared__ double2 sm[];
     const RhsBody B = bodies[blockIdx.x];
-    const int r0 = blockIdx.y * RB, nr = min(RB, nrhs - r0);
+    const int r0 = blockIdx.y * rb, nr = min(rb, nrhs - r0);
     const int m = B.m, n = B.n, k = B.k;
-    double2* t = sm;                      // [RB][m]; later C q_mfs
-    double2* qm = sm + (int64_t)RB * mmax;  // [RB][n]
-    double2* z = qm + (int64_t)RB * nmax;   // [RB][n]
+    double2* t = sm;                      // [rb][m]; later C q_mfs
+    double2* qm = sm + (int64_t)rb * mmax;  // [rb][n]
+    double2* z = qm + (int64_t)rb * nmax;   // [rb][n]
     each_entry(m, nr, [&](int i, int r) { t[(int64_t)r * m + i] = v[(int64_t)(r0 + r) * Mtot + B.voff + i]; });
     __syncthreads();
     if (B.W) {  // injected W: b = W v
@@ -1117,17 +1117,17 @@ __global__ void __launch_bounds__(32 * RB) rhs_block_kernel(const RhsBody* __res
 }
 
 __global__ void __launch_bounds__(32 * RB) recon_block_kernel(const RhsBody* __restrict__ bodies, const int nrhs,
-                                                              const int mmax, const int nmax,
+                                                              const int rb, const int mmax, const int nmax,
                                                               const double2* __restrict__ v, const int64_t Mtot,
                                                               const double2* __restrict__ w_hat, const int64_t N,
                                                               double2* __restrict__ qmfs, const int64_t Nm) {
     extern __shared__ double2 sm[];
     const RhsBody B = bodies[blockIdx.x];
-    const int r0 = blockIdx.y * RB, nr = min(RB, nrhs - r0);
+    const int r0 = blockIdx.y * rb, nr = min(rb, nrhs - r0);
     const int m = B.m, n = B.n, k = B.k;
     double2* t = sm;
-    double2* qm = sm + (int64_t)RB * mmax;
-    double2* z = qm + (int64_t)RB * nmax;
+    double2* qm = sm + (int64_t)rb * mmax;
+    double2* z = qm + (int64_t)rb * nmax;
     each_entry(m, nr, [&](int i, int r) {
         double2 s = v[(int64_t)(r0 + r) * Mtot + B.voff + i];
         const double2* wh = w_hat + (int64_t)(r0 + r) * N + B.boff;
@@ -1192,15 +1192,31 @@ void launch_sbuild(int dim, SBuildJob* d_jobs, int njobs, int* d_counter, int ro
     launch_phase(sbuild_phase3_kernel, njobs, team, threads, (size_t)0, st, d_jobs, njobs, d_counter + 2, team, rcond);
 }
 
+// Right-hand sides per CTA of the blocked kernels; 0 where the general ones are
+// faster.  A CTA takes 260 us for one right-hand side of 128 points and 640 us
+// for 8, alone on its SM; so few bodies get as few per CTA as still find an SM
+// each (the general kernel: 315 us a round of CTAs), many bodies 8 (1000 bodies,
+// 8 right-hand sides: 4.2 ms, general 10.6; but 1 right-hand side: 1.58 ms, 1.48).
+// Of 256 points: 770 and 2190 us against 640, so only many bodies with 4 or more
+// right-hand sides gain (200 bodies, 8: 4.3 ms, general 5.5).
+static int rhs_per_cta(int T, int nrhs, int mmax) {
+    if (mmax > 32 * RB_GROUPS) return 0;
+    const int64_t sms = mbs_num_sms(), all = (int64_t)T * nrhs;
+    if (mmax > 128) return nrhs >= 4 && all >= 4 * sms ? RB : 0;
+    for (int rb = 1; rb < RB; rb *= 2)
+        if ((int64_t)T * ((nrhs + rb - 1) / rb) <= sms) return rb;
+    return nrhs > 1 ? std::min(RB, nrhs) : 0;
+}
+
 void launch_rhs(const RhsBody* d_bodies, int T, int nrhs, int mmax, int nmax, const double2* v,
                 int64_t Mtot, double2* b, int64_t N, cudaStream_t st) {
     if (T == 0 || nrhs == 0) return;
-    if (mmax <= 32 * RB_GROUPS) {
-        const size_t smb = (size_t)RB * (mmax + 2 * nmax) * sizeof(double2);
+    if (const int rb = rhs_per_cta(T, nrhs, mmax)) {
+        const size_t smb = (size_t)rb * (mmax + 2 * nmax) * sizeof(double2);
         if (smb > 48 * 1024)
             MBS_CUDA_TRY(cudaFuncSetAttribute(rhs_block_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smb));
-        const dim3 gb((unsigned)T, (unsigned)((nrhs + RB - 1) / RB));
-        rhs_block_kernel<<<gb, 32 * RB, smb, st>>>(d_bodies, nrhs, mmax, nmax, v, Mtot, b, N);
+        const dim3 gb((unsigned)T, (unsigned)((nrhs + rb - 1) / rb));
+        rhs_block_kernel<<<gb, 32 * RB, smb, st>>>(d_bodies, nrhs, rb, mmax, nmax, v, Mtot, b, N);
         MBS_CHECK_LAUNCH();
         return;
     }
@@ -1217,12 +1233,12 @@ void launch_recon(const RhsBody* d_bodies, int T, int nrhs, int mmax, int nmax, 
                   int64_t Mtot, const double2* w_hat, int64_t N, double2* qmfs, int64_t Nm,
                   cudaStream_t st) {
     if (T == 0 || nrhs == 0) return;
-    if (mmax <= 32 * RB_GROUPS) {
-        const size_t smb = (size_t)RB * (mmax + 2 * nmax) * sizeof(double2);
+    if (const int rb = rhs_per_cta(T, nrhs, mmax)) {
+        const size_t smb = (size_t)rb * (mmax + 2 * nmax) * sizeof(double2);
         if (smb > 48 * 1024)
             MBS_CUDA_TRY(cudaFuncSetAttribute(recon_block_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smb));
-        const dim3 gb((unsigned)T, (unsigned)((nrhs + RB - 1) / RB));
-        recon_block_kernel<<<gb, 32 * RB, smb, st>>>(d_bodies, nrhs, mmax, nmax, v, Mtot, w_hat, N, qmfs, Nm);
+        const dim3 gb((unsigned)T, (unsigned)((nrhs + rb - 1) / rb));
+        recon_block_kernel<<<gb, 32 * RB, smb, st>>>(d_bodies, nrhs, rb, mmax, nmax, v, Mtot, w_hat, N, qmfs, Nm);
         MBS_CHECK_LAUNCH();
         return;
     }
