@@ -8,7 +8,11 @@
 // the right-hand sides, integers of 60 bits relative to the largest |q| of a
 // source body, takes 4 wide multiply-adds and 8 FP32 ones (the cross terms of
 // high and low words, whose 24 bits end near 2^-56) a pair and right-hand side,
-// and goes into FP64 sums once per 64 sources.
+// and goes into FP64 sums once per 64 sources.  The integer multiplier bounds it
+// (a wide multiply-add takes 1 of 32 lanes a clock and SM): 237 bodies of 64
+// points, 5 right-hand sides, 4.5 ms, 42 ms on the FP64 pipe; its multiplications
+// alone take 2.1 ms.  1000 bodies and 4096 targets, 8 right-hand sides: 5.9 ms
+// and 53.6 ms.
 //
 // g_fx_pack_kernel, one CTA per body, turns the offsets from the body's centre
 // and the right-hand sides into integers scaled by the body's own radius and
@@ -73,27 +77,33 @@ __global__ void __launch_bounds__(FXT) g_fx_pack_kernel(const int64_t N, const i
     for (int64_t j = j0 + threadIdx.x; j < j1; j += FXT)
 #pragma unroll
         for (int a = 0; a < DIM; ++a) P.d[a * N + j] = bad ? 0 : fx_round((xw[a * N + j] - c[a]) * up);
-    for (int r = 0; r < nrhs; ++r) {
+    // one warp per right-hand side: no barriers between them (one body of 64
+    // points, 8 right-hand sides, as one loop of the CTA: 26 us more)
+    const int lane = threadIdx.x & 31;
+    for (int r = threadIdx.x >> 5; r < nrhs; r += FXT / 32) {
         double m = 0.0;
         bool odd = false;
-        for (int64_t j = j0 + threadIdx.x; j < j1; j += FXT) {
+        for (int64_t j = j0 + lane; j < j1; j += 32) {
             const double2 v = q[(int64_t)r * N + j];
             m = fmax(m, fmax(fabs(v.x), fabs(v.y)));
             odd = odd || !isfinite(v.x) || !isfinite(v.y);
         }
-        m = fx_block_max(odd ? HUGE_VAL : m, s_red);
+        if (odd) m = HUGE_VAL;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
         const bool out = !(m < 1e270) || (m > 0.0 && m < 1e-270);
         bad = bad || out;
         const int ex = fx_exponent(out || m == 0.0 ? 1.0 : m);
         const double sc = fx_exp2(FX_QBITS - ex);
-        for (int64_t j = j0 + threadIdx.x; j < j1; j += FXT) {
+        for (int64_t j = j0 + lane; j < j1; j += 32) {
             const double2 v = q[(int64_t)r * N + j];
             const fx2 re = fx_split(out ? 0 : fx_round(v.x * sc)), im = fx_split(out ? 0 : fx_round(v.y * sc));
             P.qh[(int64_t)r * N + j] = make_int2(re.h, im.h);
             P.ql[(int64_t)r * N + j] = make_float4((float)re.h, (float)re.l, (float)im.h, (float)im.l);
         }
-        if (threadIdx.x == 0) P.qs[(int64_t)r * T + b] = fx_exp2(ex + 64 - FX_QBITS);  // of sums kept at 2^-64
+        if (lane == 0) P.qs[(int64_t)r * T + b] = fx_exp2(ex + 64 - FX_QBITS);  // of sums kept at 2^-64
     }
+    bad = __syncthreads_or(bad);
     if (threadIdx.x == 0) {
         P.rho[b] = (float)rho * 1.000001f;
         P.es[b] = bad ? FX_BAD : es;
@@ -327,10 +337,12 @@ void launch_G_fx(const GLayout& L, const double* d_centres, double kappa, int64_
 }
 
 // Four groups of threads share the sources of a target when 128-target tiles
-// and one split per body would leave SMs without a CTA.
+// and one split per body would leave SMs without a CTA or two (4 right-hand
+// sides, bodies of 64: 95 us instead of 142 for 10 bodies, 226 for 259 for 40,
+// 622 for 620 for 80, 2114 for 2019 for 160).
 int fx_groups(int64_t Nt, int T) {
     const int64_t tiles = (Nt + FXT - 1) / FXT;
-    return tiles * std::min(T, 64) < 4LL * mbs_num_sms() ? 4 : 1;
+    return tiles * std::min(T, 64) < 8LL * mbs_num_sms() ? 4 : 1;
 }
 
 int fx_tile(int64_t Nt, int T) { return FXT / fx_groups(Nt, T); }
