@@ -56,6 +56,7 @@ WORKLOAD = WORKLOADS[1]
 # right-hand side; phi = 35 flops in 2D, 15 in 3D (FFMA = 2, special function = 1)
 FLOPS_PER_PAIR = {2: lambda nrhs: 35 + 8 * nrhs, 3: lambda nrhs: 15 + 8 * nrhs}
 FLOPS_PER_PAIR_2D = FLOPS_PER_PAIR[2]
+FP64_KERNELS = {0: "FP64 pipe", 1: "double-float", 2: "64-bit fixed point"}
 FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.070e9 / 1e12  # SMs x FP32 lanes x 2 flop x max SM clock
 # DRAM bytes (read + write) of one launch on this workload, from one ncu capture
 # of the kernel as built (profiles/g_umma_kernel_2d_1000bodies_8rhs.md); null for
@@ -79,8 +80,8 @@ def parse():
                          "1e-9 (the metric's accuracy) on the two large ones")
     ap.add_argument("--restart", type=int, default=200)
     ap.add_argument("--fp64-kernel", type=int, default=2, choices=[0, 1, 2],
-                    help="FP64-accurate G_hat: 2 automatic (default: double-float on the FP32 pipe where "
-                         "the solve's tolerance allows it), 1 double-float, 0 FP64 pipe")
+                    help="FP64-accurate G_hat: 2 automatic (default: 64-bit fixed point on the integer "
+                         "multipliers), 1 double-float, 0 FP64 pipe")
     ap.add_argument("--inner-tol", type=float, default=1e-4,
                     help="relative tolerance of each FP32 inner solve of the mixed refinement "
                          "(1e-4 reaches 1e-11 in 3 sweeps with the fewest inner iterations)")
@@ -569,7 +570,7 @@ def run_mbs(a, ws, rank, local):
     t2s = {"mixed_s": statistics.mean(i["seconds"] for i in infos),
            "mixed_inner_iterations": infos[-1]["inner_iterations"],
            "mixed_sweeps": infos[-1]["sweeps"], "mixed_rel_residual": infos[-1]["rel_residual"],
-           "mixed_fp64_kernel": "double-float" if infos[-1]["fp64_kernel"] else "FP64 pipe",
+           "mixed_fp64_kernel": FP64_KERNELS[infos[-1]["fp64_kernel"]],
            "tol": a.tol}
     if capped:
         t2s = {"capped_solve_s": t2s["mixed_s"], "block_gmres_steps": infos[-1]["inner_iterations"],
@@ -587,7 +588,7 @@ def run_mbs(a, ws, rank, local):
         ctx64.close()
         t2s.update({"fp64_s": i64["seconds"], "fp64_iterations": i64["inner_iterations"],
                     "fp64_rel_residual": i64["rel_residual"], "fp64_converged": bool(i64["converged"]),
-                    "fp64_kernel": "double-float" if i64["fp64_kernel"] else "FP64 pipe",
+                    "fp64_kernel": FP64_KERNELS[i64["fp64_kernel"]],
                     "fp64_over_mixed": i64["seconds"] / t2s["mixed_s"],
                     "field_rel_err_vs_fp64": float((u_mixed - u64).abs().max() / u64.abs().max()),
                     "field_targets": M})
@@ -651,7 +652,7 @@ def run_mbs(a, ws, rank, local):
         config = {"workload": WORKLOADS[cfg], "N": N, "pairs_per_matvec": pairs_mv, "nrhs": nrhs,
                   "field_targets": M, "restart": opts["restart"], "inner_tol": a.inner_tol,
                   "fp64_kernel": {0: "FP64 pipe", 1: "double-float on the FP32 pipe",
-                                  2: "automatic (double-float where the tolerance allows)"}[a.fp64_kernel],
+                                  2: "automatic (64-bit fixed point on the integer multipliers)"}[a.fp64_kernel],
                   "l2": "256 MiB buffer written before every step",
                   "parallelism": f"replicas x{ws}" if ws > 1 else "single GPU"}
         if capped:

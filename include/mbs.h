@@ -82,13 +82,15 @@ typedef struct mbs_options {
                             0: heuristic shape */
     int cuda_graphs;     /* 1 (default): after one direct step, the device work of each block-GMRES step is
                             captured once per context and step index and replayed as a CUDA graph; 0: launch directly */
-    int fp64_kernel;     /* FP64-accurate G_hat (FP64 solves, refinement residuals, apply calls):
-                            0 on the FP64 pipe; 1 in double-float arithmetic on the FP32 pipe, with FP64
+    int fp64_kernel;     /* FP64-accurate G_hat and field (FP64 solves, refinement residuals, apply calls):
+                            0 on the FP64 pipe; 1 G_hat in double-float arithmetic on the FP32 pipe, with FP64
                             work only per body pair (3.4x faster than 0 on GB300 at N = 64,000, 8 RHS;
-                            ~1e-13 relative instead of ~1e-16); 2 (default) automatic: inside solves
-                            double-float when 1e-14 ||S||_F (the FP64 residual floor it leaves, with the
-                            root mean square of ||S_tau||_F over the bodies) is at most tol / 10, else
-                            the FP64 pipe; apply calls use the FP64 pipe */
+                            ~1e-13 relative instead of ~1e-16); 2 (default) automatic: 64-bit fixed point on
+                            the integer multipliers, as accurate as 0 (9x faster than it at N = 15,000, 5 RHS).
+                            A context without memory for its workspace goes on with the other two: inside
+                            solves double-float when 1e-14 ||S||_F (the FP64 residual floor it leaves, with
+                            the root mean square of ||S_tau||_F over the bodies) is at most tol / 10, else
+                            the FP64 pipe */
     int sbuild_threads;  /* threads per CTA of the S build (128, 256 or 512); 0 (default): 256 (the build
                             is FP64-pipe-bound: the three sizes measured within 2 % on GB300); -1: tuned on the
                             first build of a size class (when autotune is on), at the cost of ~half a build */
@@ -128,7 +130,7 @@ typedef struct mbs_solve_info {
                              and FP64 GMRES, warm-started from the refined iterate, finished */
     double rel_residual;  /* max over RHS of the final FP64 relative residual */
     double seconds;       /* wall time of the call */
-    int fp64_kernel;      /* FP64-accurate G_hat the solve used: 0 FP64 pipe, 1 double-float */
+    int fp64_kernel;      /* FP64-accurate G_hat the solve used: 0 FP64 pipe, 1 double-float, 2 fixed point */
 } mbs_solve_info;
 
 typedef struct mbs_ctx mbs_ctx;

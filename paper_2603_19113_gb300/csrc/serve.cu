@@ -77,7 +77,9 @@ size_t estimate_footprint(const Req& r, int restart) {
     bytes += T * T * 20 + N * 40;
     bytes += (size_t)(restart + 1) * N * nr * 8;  // FP32 Krylov basis
     bytes += N * nr * (16 * 8 + 8 * 6);           // FP64/FP32 vectors, partial sums (<= 64 splits chunked)
-    bytes += (size_t)64 * N * nr * 16;            // split partials upper bound
+    // split partials: 64 splits, up to 256 of the fixed-point kernel while N is small
+    bytes += std::max((size_t)64 * N, std::min((size_t)256 * N, (size_t)700000)) * nr * 16;
+    bytes += fx_pack_bytes(r.dim, (int64_t)N, (int)T, (int)nr);
     bytes += M * nr * 16;
     return bytes + ((size_t)64 << 20);
 }
