@@ -520,8 +520,9 @@ Shape32 shape32(mbs_ctx* c, int nrhs, const float2* x, float2* y) {
         for (int ns : {base, base / 2, 2 * base, 4 * base}) {
             // four times the usual count: small CTAs even out bodies of uneven
             // size (700 bodies, 16 right-hand sides: 4.64 ms with 14 splits, 4.30
-            // with 28); the FP32-pipe kernel gains nothing
-            if (ns == 4 * base && p != 3) continue;
+            // with 28); the FP32-pipe kernel gains nothing, and up to 4 right-hand
+            // sides in 3D take that one (below)
+            if (ns == 4 * base && (p != 3 || (c->dim == 3 && nrhs <= 4))) continue;
             ns = std::max(1, std::min(ns, max_nsplit(c)));
             bool dup = false;
             for (const Shape32& q : cand) dup = dup || (q.path == p && q.nsplit == ns);
@@ -551,6 +552,10 @@ Shape32 shape32(mbs_ctx* c, int nrhs, const float2* x, float2* y) {
             MBS_CUDA_TRY(cudaEventElapsedTime(&t, a, b));
             ms = rep == 0 ? t : std::min(ms, t);
         }
+        // in 3D the FP32 pipe unless it is a tenth slower: its sums are 1e-6 off,
+        // the tensor cores' 5e-6 (100 ellipsoids, 4 right-hand sides: 1.39 ms
+        // and 1.41; 16: 3.3 and 1.36; in 2D both are 2e-6 off)
+        if (c->dim == 3 && cand[ci].path == 1) ms *= 0.9f;
         if (ci == 0 || ms < best_ms) {
             best_ms = ms;
             best = cand[ci];
