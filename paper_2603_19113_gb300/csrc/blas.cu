@@ -766,7 +766,7 @@ __global__ void ts_coef32_kernel(const double2* __restrict__ H, const int ka, co
 // B_b += sum_a A_a coef(a, b) (kb <= 8), the basis streamed through a ring of
 // shared-memory stages by 2D tensor copies (TMA).
 //
-// CTA x: rows [64 x, 64 x + 64), two per lane.  The copy warp (warp 4, one
+// CTA or cluster x: rows [64 x, 64 x + 64), two per lane.  The copy warp (warp 4, one
 // lane) fills stage t with those rows of basis columns 16 t .. 16 t + 15 (a
 // bca x 512-byte box of the basis's tensor map, bca = min(16, ka); rows past N and columns past
 // ka arrive as zeros) and with their FP32 coefficients (16 x 8 float2, one
@@ -774,7 +774,9 @@ __global__ void ts_coef32_kernel(const double2* __restrict__ H, const int ka, co
 // Compute warp w takes columns 16 t + 4 w .. 16 t + 4 w + 3 of every stage,
 // so its sums run over columns in order; after the last stage the four warp
 // sums are added in warp order through shared memory (the ring, by then
-// idle) and the read-modify-write of B follows.  Waits are bounded as in the
+// idle) and the read-modify-write of B follows.  Few row tiles are shared out
+// over clusters of CTAs (update32_team), each taking a part of the columns; the
+// first adds their sums in rank order out of the others' shared memory.  Waits are bounded as in the
 // Gram kernel.
 constexpr int RU_ROWS = 64;
 constexpr int RU_COLS = 16;
@@ -786,6 +788,42 @@ constexpr int RU_STAGE = RU_COLS * RU_COLBYTES + RU_COLS * 8 * 8;
 constexpr int RU_SMEM = RU_STAGES * RU_STAGE;
 static_assert(RU_SMEM >= RU_WARPS * 8 * 32 * 16, "the ring holds the cross-warp reduction");
 
+__device__ __forceinline__ int cluster_size() {
+    int n;
+    asm("mov.u32 %0, %cluster_nctarank;" : "=r"(n));
+    return n;
+}
+
+__device__ __forceinline__ int cluster_rank() {
+    int n;
+    asm("mov.u32 %0, %cluster_ctarank;" : "=r"(n));
+    return n;
+}
+
+// every thread of the cluster that has not returned
+__device__ __forceinline__ void cluster_arrive_wait() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// the float4 at this CTA's shared address in CTA m of the cluster
+__device__ __forceinline__ float4 peer_float4(uint32_t addr, int m) {
+    uint32_t p;
+    float4 v;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(p) : "r"(addr), "r"(m));
+    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                 : "r"(p)
+                 : "memory");
+    return v;
+}
+
+__device__ __forceinline__ void add4(float4& a, const float4 b) {
+    a.x += b.x;
+    a.y += b.y;
+    a.z += b.z;
+    a.w += b.w;
+}
+
 __global__ void __launch_bounds__(RU_THREADS, 7) ts_update32_kernel(const __grid_constant__ CUtensorMap tmA,
                                                                    const int ka, const int bca,
                                                                    const float2* __restrict__ coef,
@@ -796,9 +834,11 @@ __global__ void __launch_bounds__(RU_THREADS, 7) ts_update32_kernel(const __grid
     __shared__ __align__(8) uint64_t empty[RU_STAGES];
     __shared__ volatile int s_abort;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t r0 = (int64_t)blockIdx.x * RU_ROWS;
+    const int team = cluster_size(), rank = cluster_rank();
+    const int64_t r0 = (int64_t)(blockIdx.x / team) * RU_ROWS;
     const int rows = (int)min((int64_t)RU_ROWS, N - r0);
-    const int nst = (ka + RU_COLS - 1) / RU_COLS;
+    const int all = (ka + RU_COLS - 1) / RU_COLS, t0 = (int)((int64_t)all * rank / team);
+    const int nst = (int)((int64_t)all * (rank + 1) / team) - t0;
     const uint32_t sbase = smem_u32(ru_smem);
     if (sbase & 127u) {  // tensor copies need 128-byte aligned stages: report, copy nothing
         if (threadIdx.x == 0) atomicExch(err, 1);
@@ -836,7 +876,7 @@ __global__ void __launch_bounds__(RU_THREADS, 7) ts_update32_kernel(const __grid
                 }
             }
             if (lane == 0) {
-                const int c0 = t * RU_COLS, cols = min(RU_COLS, ka - c0);
+                const int c0 = (t0 + t) * RU_COLS, cols = min(RU_COLS, ka - c0);
                 const uint32_t fb = smem_u32(&full[s]);
                 const uint32_t st = sbase + (uint32_t)(s * RU_STAGE);
                 mbar_arrive_expect(fb, (uint32_t)(bca * RU_COLBYTES + cols * 64));
@@ -899,31 +939,38 @@ __global__ void __launch_bounds__(RU_THREADS, 7) ts_update32_kernel(const __grid
 #pragma unroll
     for (int b = 0; b < 8; ++b) red[(warp * 8 + b) * 32 + lane] = make_float4(acc[b][0], acc[b][1], acc[b][2], acc[b][3]);
     asm volatile("bar.sync 1, %0;" ::"n"(RU_WARPS * 32) : "memory");
-    const bool abort = s_abort != 0;
+    // column b's sum over the warps, in warp order: thread b * 32 + lane and the
+    // next 128; a team's in rank order, by its first CTA
+    const float nanv = __int_as_float(0x7fc00000);
+    float4 tsum[8 / RU_WARPS];
+#pragma unroll
+    for (int k = 0; k < 8 / RU_WARPS; ++k) {
+        const int b = warp * (8 / RU_WARPS) + k;
+        tsum[k] = red[b * 32 + lane];
+#pragma unroll
+        for (int w = 1; w < RU_WARPS; ++w) add4(tsum[k], red[(w * 8 + b) * 32 + lane]);
+        if (s_abort) tsum[k] = make_float4(nanv, nanv, nanv, nanv);
+    }
+    if (team > 1) {
+#pragma unroll
+        for (int k = 0; k < 8 / RU_WARPS; ++k)  // each thread's own entries: no other reads them
+            red[(warp * (8 / RU_WARPS) + k) * 32 + lane] = tsum[k];
+        cluster_arrive_wait();
+        if (rank == 0)
+            for (int m = 1; m < team; ++m)
+#pragma unroll
+                for (int k = 0; k < 8 / RU_WARPS; ++k)
+                    add4(tsum[k], peer_float4(smem_u32(red + (warp * (8 / RU_WARPS) + k) * 32 + lane), m));
+        cluster_arrive_wait();  // every CTA's sums stay until the first has read them
+        if (rank > 0) return;
+    }
 #pragma unroll
     for (int k = 0; k < 8 / RU_WARPS; ++k) {
         const int b = warp * (8 / RU_WARPS) + k;
         if (b < kb && live) {
-            float4 tsum = red[b * 32 + lane];
-#pragma unroll
-            for (int w = 1; w < RU_WARPS; ++w) {
-                const float4 u = red[(w * 8 + b) * 32 + lane];
-                tsum.x += u.x;
-                tsum.y += u.y;
-                tsum.z += u.z;
-                tsum.w += u.w;
-            }
             float4* o = reinterpret_cast<float4*>(B + (int64_t)b * N + r0 + 2 * lane);
             float4 x = *o;
-            if (abort) {
-                const float nanv = __int_as_float(0x7fc00000);
-                x = make_float4(nanv, nanv, nanv, nanv);
-            } else {
-                x.x += tsum.x;
-                x.y += tsum.y;
-                x.z += tsum.z;
-                x.w += tsum.w;
-            }
+            add4(x, tsum[k]);
             *o = x;
         }
     }
@@ -1188,6 +1235,19 @@ void launch_ts_gram(const V* A, int ka, const V* B, int kb, int64_t N, double2* 
     MBS_CHECK_LAUNCH();
 }
 
+// CTAs that share a row tile's basis columns (a cluster).  With about one CTA an
+// SM a scheduler has one warp, which issues every fourth clock, and SMs with two
+// CTAs are done last; halves and quarters of the columns fill the SMs and even
+// them out, until there are enough tiles (a solve's step less its operator, 8
+// right-hand sides, with 1, 2, 4, 8 CTAs a tile: 160 tiles and up to 1600 columns
+// 214, 195, 188, 196 us; 300 tiles and up to 800 columns 173, 168, 176, 188; 450:
+// 202, 200, 211, 229; 600: 224, 230, 238, 257).  Every CTA keeps its ring busy.
+static int update32_team(int64_t tiles, int ka) {
+    int team = 2 * tiles <= 3 * mbs_num_sms() ? 4 : tiles <= 3 * mbs_num_sms() ? 2 : 1;
+    while (team > 1 && ka < 4 * RU_COLS * team) team /= 2;
+    return team;
+}
+
 template <typename V>
 void launch_ts_update(const V* A, int ka, const double2* H, double alpha, V* B, int kb, int64_t N,
                       cudaStream_t st, float2* coef, int* err) {
@@ -1202,8 +1262,21 @@ void launch_ts_update(const V* A, int ka, const double2* H, double alpha, V* B, 
         ring_smem_attr(ts_update32_kernel, RU_SMEM, g_update_attr);
         const int bca = std::min(RU_COLS, ka);
         const CUtensorMap tmA = column_map(A, N, ka, bca);
-        ts_update32_kernel<<<(unsigned)((N + RU_ROWS - 1) / RU_ROWS), RU_THREADS, RU_SMEM, st>>>(
-            tmA, ka, bca, coef, reinterpret_cast<float2*>(B), kb, N, err);
+        const int64_t tiles = (N + RU_ROWS - 1) / RU_ROWS;
+        const int team = update32_team(tiles, ka);
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3((unsigned)(tiles * team));
+        cfg.blockDim = dim3(RU_THREADS);
+        cfg.dynamicSmemBytes = RU_SMEM;
+        cfg.stream = st;
+        cudaLaunchAttribute at{};
+        at.id = cudaLaunchAttributeClusterDimension;
+        at.val.clusterDim.x = (unsigned)team;
+        at.val.clusterDim.y = at.val.clusterDim.z = 1;
+        cfg.attrs = &at;
+        cfg.numAttrs = team > 1 ? 1 : 0;
+        MBS_CUDA_TRY(cudaLaunchKernelEx(&cfg, ts_update32_kernel, tmA, ka, bca, (const float2*)coef,
+                                        reinterpret_cast<float2*>(B), kb, N, err));
     } else if (kb <= 8) {
         ts_update_kernel<V, 8><<<nblocks(N), 256, 0, st>>>(A, ka, H, alpha, B, kb, N);
     } else {

@@ -1,6 +1,7 @@
 """GPU kernels beside the general ones: the fixed-point sums (gfixed.cu), the
-S build shared out over clusters, the blocked right-hand side, and the sorting
-of targets to proxies, at the sizes where each can go wrong."""
+S build shared out over clusters, the blocked right-hand side, the sorting of
+targets to proxies and the Gram-Schmidt updates on clusters, at the sizes where
+each can go wrong."""
 import numpy as np
 import pytest
 
@@ -218,3 +219,20 @@ def test_targets_are_sorted_to_proxies(pkg, dim, M):
     o = int(np.sum(n_of[:2]))
     ref = K @ q + orc.kernel_matrix(dim, wl.kappa, near[i:i + 1], wl.body_points(2, "y")) @ qm[o:o + n_of[2]]
     assert _rel(un[i:i + 1], ref) < 1e-12
+
+
+@pytest.mark.parametrize("T,ks", [(30, (24, 36, 50)), (300, (50,)), (460, (64,))])
+def test_basis_update_teams(pkg, T, ks):
+    """Mixed solves whose Gram-Schmidt updates run on clusters of 4, 2 and 1 CTAs
+    per row tile (16 rows ragged, and bases from one column block up): the residual
+    the solver reports is the one its FP64 operator shows, and refinement contracts
+    as an exact Arnoldi relation lets it."""
+    wl = mi.tiny_2d(seed=6, T=T, kappa=12.0, nrhs=8, ks=ks)
+    with pkg.Context(2, wl.kappa, precision=pkg.PREC_MIXED, tol=1e-11, restart=100) as ctx:
+        ctx.build_scattering_matrices(wl)
+        b = ctx.rhs(wl.boundary_data())
+        q, info = ctx.solve(b)
+        assert info["converged"] == 1 and info["fp64_finish"] == 0 and info["sweeps"] <= 4
+        ctx.set_options(precision=pkg.PREC_FP64)
+        r = b - ctx.apply_operator(q)
+        assert np.max(np.linalg.norm(r, axis=0) / np.linalg.norm(b, axis=0)) < 1e-11 * 1.01
