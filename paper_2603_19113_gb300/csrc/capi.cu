@@ -406,7 +406,7 @@ int* device_err(mbs_ctx* c) {
 // power-of-two buckets of N and of the body count) times every candidate
 // shape on the caller's own data: the kernel path (tcgen05 or FP32 pipe,
 // unless mac_path fixes it) times the source-split count (the heuristic's,
-// half and double).  The fastest is kept in a process-wide table, so every
+// half, double and four times it).  The fastest is kept in a process-wide table, so every
 // later matvec of that class, in any context, uses the same shape; a solve
 // therefore gives the same result alone and next to other solves.
 // mbs_options.autotune = 0 (or a tile_override) keeps the heuristic shape.

@@ -2,10 +2,9 @@
 // accuracy in 64-bit fixed point on the integer multipliers.  Host and device
 // code.
 //
-// GB300 issues 62 32x32+64-bit integer multiply-adds per clock and SM
-// (IMAD.WIDE, measured) and 2 FP64 ones, so a 64 x 64 -> 64 (high half)
-// product from three of them costs a tenth of one FP64 multiply-add and keeps
-// more bits.  Distances are taken relative to one source body: with its
+// GB300 does 32 32x32+64-bit integer multiply-adds per clock and SM (measured)
+// and 2 FP64 ones, so a 64 x 64 -> 64 (high half) product from three of them
+// costs a fifth of one FP64 multiply-add and keeps more bits.  Distances are taken relative to one source body: with its
 // reference point c, radius rho and a target t, D = t - c (FP64, once per
 // target and body) and 2^e > |D| + rho, every length is a fraction of 2^e in
 // [0, 1) with 62 bits, so the phase kappa r carries 2^-62 kappa 2^e, against
