@@ -8,11 +8,12 @@
 // the right-hand sides, integers of 60 bits relative to the largest |q| of a
 // source body, takes 4 wide multiply-adds and 8 FP32 ones (the cross terms of
 // high and low words, whose 24 bits end near 2^-56) a pair and right-hand side,
-// and goes into FP64 sums once per 64 sources.  The integer multiplier bounds it
-// (a wide multiply-add takes 1 of 32 lanes a clock and SM): 237 bodies of 64
-// points, 5 right-hand sides, 4.5 ms, 42 ms on the FP64 pipe; its multiplications
-// alone take 2.1 ms.  1000 bodies and 4096 targets, 8 right-hand sides: 5.9 ms
-// and 53.6 ms.
+// and goes into FP64 sums once per 64 sources.  237 bodies of 64
+// points, 5 right-hand sides: 4.35 ms, 42 ms on the FP64 pipe; 1000 bodies and
+// 4096 targets, 8 right-hand sides: 5.7 ms and 53.6 ms.  The wide multiply-adds
+// alone, 32 a clock and SM, would take 2.1 ms of the 4.35; issue slots are 57 %
+// busy, the ALU 52 %, and warps wait for dispatch, busy pipes and dependent
+// results in about equal parts.
 //
 // g_fx_pack_kernel, one CTA per body, turns the offsets from the body's centre
 // and the right-hand sides into integers scaled by the body's own radius and
@@ -118,9 +119,11 @@ __device__ __noinline__ double2 fx_phi_f64(double kappa, double r2) {
 
 // One thread per target; SG groups of FXT / SG threads take SG-th parts of the
 // staged sources of the same targets (small problems, where the sources of a
-// body would otherwise be one long chain per thread).
+// body would otherwise be one long chain per thread).  4 CTAs per SM with two
+// sources in flight a thread: 5 with one source 3 % slower (4.50 ms, 237 bodies, 5
+// right-hand sides), 5 with two 2 %, 6 with one 4 % (8 right-hand sides: 12 %).
 template <int DIM, int NR, int SG>
-__global__ void __launch_bounds__(FXT, 5)
+__global__ void __launch_bounds__(FXT, 4)
     g_fx_kernel(const FxKappa kap, const int64_t Nt, const double* __restrict__ tgt, const int* __restrict__ tbody,
                 const int64_t N, const int T, const double* __restrict__ xw, const int64_t* __restrict__ off,
                 const double* __restrict__ centres, const FxPacked P, const int nrhs, const int r0,
@@ -199,7 +202,7 @@ __global__ void __launch_bounds__(FXT, 5)
             const int part_n = (n + SG - 1) / SG;
             const int k0 = grp * part_n, k1 = min(n, k0 + part_n);
             if (fast) {
-#pragma unroll 1
+#pragma unroll 2
                 for (int j = k0; j < k1; ++j) {
                     fx_i64 pr, pi;
                     if (!fx_phi<DIM>(B, s_d[j], s_tab, pr, pi)) {  // 2D, kappa r < 4
