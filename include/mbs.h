@@ -25,7 +25,11 @@
  *    the current device; the library tells them apart with
  *    cudaPointerGetAttributes.  Host buffers are copied in and out inside the
  *    call; device buffers are used in place on the context's stream, and the
- *    call returns after the stream has finished with them.
+ *    call returns after the stream has finished with them.  A stream that the
+ *    context created first waits for the legacy default stream; work on other
+ *    streams, or with options.stream on any other than that one, the caller
+ *    orders (the field calls wait for the default stream on either, as soon
+ *    as their targets are in device memory).
  *  - The caller keeps ownership of every buffer it passes; the library copies
  *    what it needs.  The library owns the context and all device memory it
  *    allocates; mbs_destroy releases it.

@@ -132,6 +132,7 @@ class Context:
         self.dim = dim
         self.kappa = kappa
         self.options = opt
+        self._stream = opt.stream or 0  # 0: the context's own
         self.N = 0
         self.T = 0
 
@@ -161,9 +162,22 @@ class Context:
         for k, v in kw.items():
             setattr(self.options, k, v)
         self._check(_lib().mbs_set_options(self._h, C.byref(self.options)))
+        self._stream = self.options.stream or self._stream
 
     def last_error(self) -> str:
         return _lib().mbs_last_error(self._h).decode()
+
+    def _ready(self, *tensors):
+        """Called last before the library takes CUDA tensors: waits for torch's
+        current stream, on which they and their copies may still be in the
+        making, unless the context's stream follows it by itself (its own stream
+        follows the default one, a caller's follows itself)."""
+        for t in tensors:
+            if _is_torch(t) and t.is_cuda:
+                s = torch.cuda.current_stream(t.device)
+                if s.cuda_stream != self._stream:
+                    s.synchronize()
+                return
 
     # ---- the paper's calls ------------------------------------------------
     def build_scattering_matrices(self, wl):
@@ -212,18 +226,21 @@ class Context:
     def rhs(self, v):
         a = _Arg(v, self.Mtot)
         out, p = _out_like(a, self.N)
+        self._ready(out)
         self._check(_lib().mbs_rhs(self._h, a.nrhs, a.ptr, p))
         return _ret(out, a)
 
     def apply_operator(self, q):
         a = _Arg(q, self.N)
         out, p = _out_like(a, self.N)
+        self._ready(out)
         self._check(_lib().mbs_apply_operator(self._h, a.nrhs, a.ptr, p))
         return _ret(out, a)
 
     def apply_G(self, q, precision: int = PREC_FP64):
         a = _Arg(q, self.N)
         out, p = _out_like(a, self.N)
+        self._ready(out)
         self._check(_lib().mbs_apply_G(self._h, precision, a.nrhs, a.ptr, p))
         return _ret(out, a)
 
@@ -243,6 +260,7 @@ class Context:
             xa = _Arg(x0, self.N)
             x = xa.keep.clone() if xa.torch else xa.keep.copy()
             xp = C.c_void_p(x.data_ptr() if xa.torch else x.ctypes.data)
+        self._ready(x, a.keep)
         info = L.mbs_solve_info()
         st = _lib().mbs_solve(self._h, a.nrhs, a.ptr, xp, C.byref(info))
         if st != L.MBS_OK and (raise_on_noconv or st != 5):
@@ -264,6 +282,7 @@ class Context:
             pp = C.c_void_p(P.ctypes.data)
             M = np.asarray(pts).shape[0]
         out, p = _out_like(a, M)
+        self._ready(out, P)
         self._check(_lib().mbs_evaluate_field(self._h, a.nrhs, M, pp, a.ptr, p))
         return _ret(out, a)
 
@@ -273,6 +292,7 @@ class Context:
         a = _Arg(v, self.Mtot)
         qa = _Arg(qhat, self.N)
         out, p = _out_like(a, self.Nm)
+        self._ready(out, qa.keep)
         self._check(_lib().mbs_reconstruct(self._h, a.nrhs, a.ptr, qa.ptr, p))
         return _ret(out, a)
 
@@ -292,6 +312,7 @@ class Context:
             pp = C.c_void_p(P.ctypes.data)
             M = np.asarray(pts).shape[0]
         out, p = _out_like(a, M)
+        self._ready(out, P, ma.keep)
         self._check(_lib().mbs_evaluate_field_near(self._h, a.nrhs, M, pp, a.ptr, ma.ptr, p))
         return _ret(out, a)
 

@@ -62,6 +62,8 @@ struct mbs_ctx {
     mbs_options opt{};
     cudaStream_t st = nullptr;
     bool own_stream = false;
+    cudaEvent_t caller = nullptr;  // on the legacy default stream: the caller's work on device arguments
+    bool ordered = false;          // this call waits for it
     std::mutex mu;
     std::string err;
 
@@ -256,15 +258,33 @@ bool is_device_ptr(const void* p) {
     return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
+// The context's work from here on follows what the legacy default stream holds:
+// device arguments may still be in the making there, and the context's own
+// stream, which does not wait for it by itself, is not known to the caller.
+void after_default_stream(mbs_ctx* c) {
+    if (c->ordered) return;
+    if (!c->caller) MBS_CUDA_TRY(cudaEventCreateWithFlags(&c->caller, cudaEventDisableTiming));
+    MBS_CUDA_TRY(cudaEventRecord(c->caller, cudaStreamLegacy));
+    MBS_CUDA_TRY(cudaStreamWaitEvent(c->st, c->caller, 0));
+    c->ordered = true;
+}
+
 // Device view of a caller's complex input array (copied if it lives on the host).
 const double2* in_dev(mbs_ctx* c, const double* p, size_t ncomplex, const char* name) {
-    if (is_device_ptr(p)) return reinterpret_cast<const double2*>(p);
+    if (is_device_ptr(p)) {
+        if (c->own_stream) after_default_stream(c);
+        return reinterpret_cast<const double2*>(p);
+    }
     double2* d = scratch<double2>(c, name, ncomplex);
     MBS_CUDA_TRY(cudaMemcpyAsync(d, p, ncomplex * sizeof(double2), cudaMemcpyHostToDevice, c->st));
     return d;
 }
+// Targets: the field calls follow the default stream on a caller's stream too.
 const double* in_dev_real(mbs_ctx* c, const double* p, size_t n, const char* name) {
-    if (is_device_ptr(p)) return p;
+    if (is_device_ptr(p)) {
+        after_default_stream(c);
+        return p;
+    }
     double* d = scratch<double>(c, name, n);
     MBS_CUDA_TRY(cudaMemcpyAsync(d, p, n * sizeof(double), cudaMemcpyHostToDevice, c->st));
     return d;
@@ -278,6 +298,7 @@ struct OutBuf {
 };
 OutBuf out_dev(mbs_ctx* c, double* p, size_t ncomplex, const char* name) {
     OutBuf o{p, nullptr, ncomplex, !is_device_ptr(p)};
+    if (!o.host && c->own_stream) after_default_stream(c);  // its memory may still be in use there
     o.dev = o.host ? scratch<double2>(c, name, ncomplex) : reinterpret_cast<double2*>(p);
     return o;
 }
@@ -1258,6 +1279,7 @@ template <typename F>
 mbs_status guarded(mbs_ctx* c, F&& f) {
     if (!c) return MBS_ERR_ARG;
     std::lock_guard<std::mutex> g(c->mu);
+    c->ordered = false;
     try {
         const mbs_status s = f();
         if (c->d_err) {
@@ -1846,6 +1868,7 @@ void mbs_destroy(mbs_ctx* c) {
         c->d_err = nullptr;
         if (c->pinned) cudaFreeHost(c->pinned);
         c->pinned = nullptr;
+        if (c->caller) cudaEventDestroy(c->caller);
         if (c->own_stream && c->st) cudaStreamDestroy(c->st);
     }
     delete c;
