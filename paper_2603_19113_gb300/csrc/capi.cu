@@ -189,7 +189,7 @@ void clear_graphs(mbs_ctx* c) {
 // context whose memory or budget is exhausted goes on with the other
 // FP64-accurate kernels, which need none.
 bool drop_fx(mbs_ctx* c) {
-    auto it = c->bufs.find("fx_pack");
+    auto it = c->bufs.find("fx_work");
     if (it == c->bufs.end() || !it->second.p || c->capturing) return false;
     clear_graphs(c);
     if (c->st) cudaStreamSynchronize(c->st);
@@ -352,20 +352,6 @@ int* split_table(mbs_ctx* c, int ns) {
     MBS_CUDA_TRY(cudaMemcpy(d, sb.data(), sb.size() * sizeof(int), cudaMemcpyHostToDevice));
     c->split_cache[key] = d;
     return d;
-}
-
-// Workspace of the fixed-point kernel, the default FP64-accurate one
-// (fp64_kernel = 2); null where an option picks another kernel or there is no
-// memory for it.  Taken after every other buffer of a call (see drop_fx).
-void* fx_workspace(mbs_ctx* c, int nrhs) {
-    if (c->opt.fp64_kernel != 2 || c->fx_off) return nullptr;
-    try {
-        return scratch<unsigned char>(c, "fx_pack", fx_pack_bytes(c->dim, c->N, c->T, nrhs));
-    } catch (const MbsError& e) {
-        if (e.st != MBS_ERR_NOMEM) throw;
-        c->fx_off = true;
-        return nullptr;
-    }
 }
 
 GLayout glayout(mbs_ctx* c) {
@@ -614,27 +600,54 @@ int fx_nsplit(mbs_ctx* c, int64_t ntargets) {
     return (int)std::max<int64_t>(1, std::min<int64_t>(ns, std::min(c->T, 256)));
 }
 
-// Partial sums of the FP64-accurate kernels: for the fixed-point kernel's splits
-// where there is memory for them, at least for the others'.
-double2* part64(mbs_ctx* c, const char* name, int ns64, int nsfx, size_t len) {
-    if (nsfx > ns64) {
+// Workspace of the fixed-point kernel, the default FP64-accurate one
+// (fp64_kernel = 2): packed sources and the partial sums of its source splits,
+// in one buffer that is taken after every other one of a call and gives way to
+// all of them (drop_fx).  With little memory fewer splits; null pack where an
+// option picks another kernel or there is no memory at all.
+struct FxWork {
+    unsigned char* pack = nullptr;
+    double2* part = nullptr;
+    int nsplit = 0;
+    int* sb = nullptr;
+};
+FxWork fx_workspace(mbs_ctx* c, int64_t ntargets, int nrhs) {
+    FxWork w;
+    if (c->opt.fp64_kernel != 2 || c->fx_off) return w;
+    const size_t pack = (fx_pack_bytes(c->dim, c->N, c->T, nrhs) + 255) & ~(size_t)255;
+    const int most = fx_nsplit(c, ntargets);
+    for (int ns : {most, choose_nsplit(c, ntargets)}) {
+        if (ns > most) continue;
+        const size_t need = pack + (size_t)ns * nrhs * ntargets * sizeof(double2);
+        const size_t held = c->bufs["fx_work"].n;
+        if (need > held && (c->capturing ||
+                            (c->opt.hbm_budget && c->bytes_held - held + need > c->opt.hbm_budget)))
+            continue;
         try {
-            return scratch<double2>(c, name, nsfx * len);
+            w.sb = split_table(c, ns);
+            w.pack = scratch<unsigned char>(c, "fx_work", need);
         } catch (const MbsError& e) {
             if (e.st != MBS_ERR_NOMEM) throw;
-            c->fx_off = true;
+            continue;
         }
+        w.part = reinterpret_cast<double2*>(w.pack + pack);
+        w.nsplit = ns;
+        return w;
     }
-    return scratch<double2>(c, name, ns64 * len);
+    c->fx_off = true;
+    return FxWork{};
 }
 
 void G64(mbs_ctx* c, int nrhs, const double2* x, double2* y) {
     // one body has no pairs: the kernel without a packing launch (45 us, not 60)
-    const bool want_fx = c->opt.fp64_kernel == 2 && !c->fx_off && c->T > 1;
-    const int ns64 = choose_nsplit(c, c->N), nsfx = want_fx ? fx_nsplit(c, c->N) : 0;
-    double2* part = part64(c, "part64", ns64, nsfx, (size_t)nrhs * c->N);
-    int* sb = split_table(c, ns64);
-    int* sbfx = want_fx ? split_table(c, nsfx) : nullptr;
+    const FxWork fx = c->T > 1 ? fx_workspace(c, c->N, nrhs) : FxWork{};
+    const int ns = choose_nsplit(c, c->N);
+    double2* part = nullptr;
+    int* sb = nullptr;
+    if (!fx.pack) {
+        part = scratch<double2>(c, "part64", (size_t)ns * nrhs * c->N);
+        sb = split_table(c, ns);
+    }
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (c->profile && c->capturing) {
         e0 = c->cap_e0;
@@ -644,31 +657,31 @@ void G64(mbs_ctx* c, int nrhs, const double2* x, double2* y) {
         e1 = take_event(c);
         c->ev64.emplace_back(e0, e1);
     }
-    if (void* pack = want_fx ? fx_workspace(c, nrhs) : nullptr) {
-        launch_G_fx(glayout(c), c->d_centres, c->kappa, c->N, c->d_xw64, c->d_body, nrhs, x, y, part, nsfx, sbfx,
-                    pack, c->st, e0, e1);
+    if (fx.pack) {
+        launch_G_fx(glayout(c), c->d_centres, c->kappa, c->N, c->d_xw64, c->d_body, nrhs, x, y, fx.part, fx.nsplit,
+                    fx.sb, fx.pack, c->st, e0, e1);
         return;
     }
     if (c->opt.fp64_kernel == 1 || (c->opt.fp64_kernel == 2 && c->in_solve && c->df_active)) {
         // double-float arithmetic on the FP32 pipe (gdf.cu); the events bracket
         // the kernel passes, not the split reduction, as for the FP64 kernel
-        launch_G_df(glayout(c), c->d_centres, c->kappa, nrhs, x, y, part, ns64, sb, c->st, e0, e1);
+        launch_G_df(glayout(c), c->d_centres, c->kappa, nrhs, x, y, part, ns, sb, c->st, e0, e1);
         return;
     }
-    launch_G_f64(glayout(c), c->kappa, nrhs, x, y, part, ns64, sb, c->st, e0, e1);
+    launch_G_f64(glayout(c), c->kappa, nrhs, x, y, part, ns, sb, c->st, e0, e1);
 }
 
 // Skeleton sums at M targets (tbody nullable: per target a body left out).
 void field64(mbs_ctx* c, int nrhs, int64_t M, const double* pts, const double2* q, double2* u, const int* tbody) {
-    const bool want_fx = c->opt.fp64_kernel == 2 && !c->fx_off;
-    const int ns64 = choose_nsplit(c, M), nsfx = want_fx ? fx_nsplit(c, M) : 0;
-    double2* part = part64(c, "part_field", ns64, nsfx, (size_t)nrhs * M);
-    int* sb = split_table(c, ns64);
-    int* sbfx = want_fx ? split_table(c, nsfx) : nullptr;
-    if (void* pack = fx_workspace(c, nrhs))
-        launch_G_fx(glayout(c), c->d_centres, c->kappa, M, pts, tbody, nrhs, q, u, part, nsfx, sbfx, pack, c->st);
-    else
-        launch_field_f64(glayout(c), c->kappa, M, pts, nrhs, q, u, part, ns64, sb, c->st, tbody);
+    const FxWork fx = fx_workspace(c, M, nrhs);
+    if (fx.pack) {
+        launch_G_fx(glayout(c), c->d_centres, c->kappa, M, pts, tbody, nrhs, q, u, fx.part, fx.nsplit, fx.sb, fx.pack,
+                    c->st);
+        return;
+    }
+    const int ns = choose_nsplit(c, M);
+    double2* part = scratch<double2>(c, "part_field", (size_t)ns * nrhs * M);
+    launch_field_f64(glayout(c), c->kappa, M, pts, nrhs, q, u, part, ns, split_table(c, ns), c->st, tbody);
 }
 
 // out = x + S G_hat x
