@@ -5,6 +5,7 @@
 #include <chrono>
 #include <cmath>
 #include <complex>
+#include <cstdint>
 #include <cstring>
 #include <map>
 #include <mutex>
@@ -78,7 +79,10 @@ struct mbs_ctx {
     double snorm_rms = 0.0;  // root mean square over bodies of the Frobenius norm of S
     bool in_solve = false;
     bool df_active = false;
-    bool fx_off = false;  // no memory for the fixed-point kernel's workspace: the other FP64-accurate kernels run
+    // no memory for the fixed-point kernel's workspace: the other FP64-accurate
+    // kernels run for the rest of the call
+    bool fx_off = false;
+    size_t fx_denied = SIZE_MAX;  // size that the device had no memory for since the last build
     std::vector<int64_t> off, voff;
     std::vector<int> kb;  // per-body skeleton count
     std::vector<double> skel_world;  // dim * N SoA
@@ -228,7 +232,7 @@ void free_geometry(mbs_ctx* c) {
     c->shapes.clear();
     c->bodies.clear();
     c->built = false;
-    c->fx_off = false;
+    c->fx_denied = SIZE_MAX;
     c->T = 0;
     c->N = 0;
     c->d_body = nullptr;
@@ -620,7 +624,7 @@ FxWork fx_workspace(mbs_ctx* c, int64_t ntargets, int nrhs) {
         if (ns > most) continue;
         const size_t need = pack + (size_t)ns * nrhs * ntargets * sizeof(double2);
         const size_t held = c->bufs["fx_work"].n;
-        if (need > held && (c->capturing ||
+        if (need > held && (need >= c->fx_denied || c->capturing ||
                             (c->opt.hbm_budget && c->bytes_held - held + need > c->opt.hbm_budget)))
             continue;
         try {
@@ -628,6 +632,7 @@ FxWork fx_workspace(mbs_ctx* c, int64_t ntargets, int nrhs) {
             w.pack = scratch<unsigned char>(c, "fx_work", need);
         } catch (const MbsError& e) {
             if (e.st != MBS_ERR_NOMEM) throw;
+            c->fx_denied = std::min(c->fx_denied, need);
             continue;
         }
         w.part = reinterpret_cast<double2*>(w.pack + pack);
@@ -1293,6 +1298,7 @@ mbs_status guarded(mbs_ctx* c, F&& f) {
     if (!c) return MBS_ERR_ARG;
     std::lock_guard<std::mutex> g(c->mu);
     c->ordered = false;
+    c->fx_off = false;
     try {
         const mbs_status s = f();
         if (c->d_err) {
@@ -1902,6 +1908,7 @@ mbs_status mbs_set_options(mbs_ctx* c, const mbs_options* opt) {
         void* keep = c->opt.stream;
         clear_graphs(c);
         c->opt = *opt;
+        c->fx_denied = SIZE_MAX;
         if (!opt->stream) c->opt.stream = keep;
         return MBS_OK;
     });

@@ -1,5 +1,5 @@
 """The fixed-point kernel's workspace under a device-memory budget: optional
-memory, which refuses no call."""
+memory, which refuses no call and is taken up again when there is room."""
 import functools
 
 import numpy as np
@@ -64,3 +64,24 @@ def test_what_fits_beside_the_fp64_pipe_fits(pkg):
     least = _least(pkg, lambda b: bool(calls(b, 0)))
     for a, b in zip(calls(least + 8192, 2), calls(least, 0)):
         assert np.abs(a - b).max() < 1e-12 * np.abs(b).max()
+
+
+def test_the_workspace_comes_back(pkg):
+    """After a build that needed its memory, and with a larger budget."""
+    wl = _wl(9)
+
+    def solve(ctx):
+        return ctx.solve(_rand((ctx.N, 5), 1), raise_on_noconv=False)[1]["fp64_kernel"]
+
+    def solves(budget, builds, restart):
+        with pkg.Context(2, wl.kappa, hbm_budget=budget, restart=restart, max_iter=40) as ctx:
+            return [solve(ctx.build_scattering_matrices(wl)) for _ in range(builds)]
+
+    least = _least(pkg, lambda b: solves(b, 2, 20)[0] == 2)
+    assert solves(least, 2, 20) == [2, 2]
+    least = _least(pkg, lambda b: bool(solves(b, 1, 200)))
+    with pkg.Context(2, wl.kappa, hbm_budget=least, restart=200, max_iter=40) as ctx:
+        ctx.build_scattering_matrices(wl)
+        assert solve(ctx) != 2
+        ctx.set_options(hbm_budget=0)
+        assert solve(ctx) == 2
