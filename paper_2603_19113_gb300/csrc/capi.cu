@@ -416,7 +416,7 @@ int* device_err(mbs_ctx* c) {
 // problem class (device, dimension, right-hand sides, kernel option and the
 // power-of-two buckets of N and of the body count) times every candidate
 // shape on the caller's own data: the kernel path (tcgen05 or FP32 pipe,
-// unless mac_path fixes it) times the source-split count (the heuristic's,
+// unless mac_path fixes it), then the source-split count (the heuristic's,
 // half, double and four times it).  The fastest is kept in a process-wide table, so every
 // later matvec of that class, in any context, uses the same shape; a solve
 // therefore gives the same result alone and next to other solves.
@@ -485,21 +485,32 @@ int log2_bucket(int64_t v) {
     return b;
 }
 
+// Buffers of a launch.
+struct Work32 {
+    int* sb;
+    float2* part;
+    UmmaLayout U;
+};
+Work32 prepare_g32(mbs_ctx* c, int nrhs, const Shape32& sh) {
+    Work32 w{};
+    w.sb = split_table(c, sh.nsplit);
+    w.part = scratch<float2>(c, "part32", (size_t)sh.nsplit * nrhs * c->N);
+    if (sh.path == 3) {
+        w.U.nchunks = c->nchunks;
+        w.U.chunk_off = c->d_chunk_off;
+        w.U.chunk_body = c->d_chunk_body;
+        w.U.pack_bytes = umma_pack_bytes(c->nchunks, nrhs);
+        w.U.pack = scratch<unsigned char>(c, "umma_pack", w.U.pack_bytes);
+        w.U.err = device_err(c);
+    }
+    return w;
+}
+
 void launch_g32(mbs_ctx* c, int nrhs, const float2* x, float2* y, const Shape32& sh,
                 cudaEvent_t e0, cudaEvent_t e1) {
-    int* sb = split_table(c, sh.nsplit);
-    float2* part = scratch<float2>(c, "part32", (size_t)sh.nsplit * nrhs * c->N);
-    UmmaLayout U{};
-    if (sh.path == 3) {
-        U.nchunks = c->nchunks;
-        U.chunk_off = c->d_chunk_off;
-        U.chunk_body = c->d_chunk_body;
-        U.pack_bytes = umma_pack_bytes(c->nchunks, nrhs);
-        U.pack = scratch<unsigned char>(c, "umma_pack", U.pack_bytes);
-        U.err = device_err(c);
-    }
-    launch_G_f32(glayout(c), c->kappa, nrhs, x, y, part, sh.nsplit, sb, c->st, e0, e1, sh.path,
-                 sh.path == 3 ? &U : nullptr);
+    Work32 w = prepare_g32(c, nrhs, sh);
+    launch_G_f32(glayout(c), c->kappa, nrhs, x, y, w.part, sh.nsplit, w.sb, c->st, e0, e1, sh.path,
+                 sh.path == 3 ? &w.U : nullptr);
 }
 
 Shape32 heuristic_shape32(mbs_ctx* c, int nrhs) {
@@ -523,54 +534,64 @@ Shape32 shape32(mbs_ctx* c, int nrhs, const float2* x, float2* y) {
         sh.nsplit = std::min(sh.nsplit, max_nsplit(c));
         return sh;
     }
-    std::vector<Shape32> cand;
-    std::vector<int> paths{h.path};
-    if (c->opt.mac_path == 0 && h.path == 3) paths.push_back(1);
-    for (int p : paths) {
-        const int base = choose_nsplit(c, p == 3 ? 2 * c->N : c->N);
-        for (int ns : {base, base / 2, 2 * base, 4 * base}) {
-            // four times the usual count: small CTAs even out bodies of uneven
-            // size (700 bodies, 16 right-hand sides: 4.64 ms with 14 splits, 4.30
-            // with 28); the FP32-pipe kernel gains nothing, and up to 4 right-hand
-            // sides in 3D take that one (below)
-            if (ns == 4 * base && (p != 3 || (c->dim == 3 && nrhs <= 4))) continue;
-            ns = std::max(1, std::min(ns, max_nsplit(c)));
-            bool dup = false;
-            for (const Shape32& q : cand) dup = dup || (q.path == p && q.nsplit == ns);
-            if (!dup) cand.push_back({p, ns});
-        }
-    }
+    // The kernel path first, at the usual split counts: the other counts change
+    // times by up to a third, and what the paths' roundings differ by is not
+    // theirs to decide (3D: FP32 pipe 1e-6 off, tensor cores 5e-6).  Then the
+    // counts of that path.  All buffers and each path's first launch come before
+    // its timed ones.
     cudaEvent_t a = take_event(c), b = take_event(c);
-    Shape32 best = h;
-    float best_ms = 0.f;
-    for (size_t ci = 0; ci < cand.size(); ++ci) {
-        // an untimed launch first: the split table and the partial sums of a
-        // count are allocated by it, which took longer than a small launch and
-        // so decided the choice; launches below 0.2 ms are timed three times
+    auto time = [&](const Shape32& sh, float stop) {
         float ms = 0.f;
-        try {
-            launch_g32(c, nrhs, x, y, cand[ci], nullptr, nullptr);
-        } catch (const MbsError& e) {
-            if (e.st != MBS_ERR_NOMEM || ci == 0) throw;
-            continue;  // no memory for that many partial sums
-        }
-        for (int rep = 0; rep < 3 && (rep == 0 || ms < 0.2f); ++rep) {
+        for (int rep = 0; rep < 3 && (rep == 0 || (ms < 0.2f && ms < stop)); ++rep) {
             MBS_CUDA_TRY(cudaEventRecord(a, c->st));
-            launch_g32(c, nrhs, x, y, cand[ci], nullptr, nullptr);
+            launch_g32(c, nrhs, x, y, sh, nullptr, nullptr);
             MBS_CUDA_TRY(cudaEventRecord(b, c->st));
             MBS_CUDA_TRY(cudaEventSynchronize(b));
             float t = 0.f;
             MBS_CUDA_TRY(cudaEventElapsedTime(&t, a, b));
             ms = rep == 0 ? t : std::min(ms, t);
         }
-        // in 3D the FP32 pipe unless it is a tenth slower: its sums are 1e-6 off,
-        // the tensor cores' 5e-6 (100 ellipsoids, 4 right-hand sides: 1.39 ms
-        // and 1.41; 16: 3.3 and 1.36; in 2D both are 2e-6 off)
-        if (c->dim == 3 && cand[ci].path == 1) ms *= 0.9f;
-        if (ci == 0 || ms < best_ms) {
-            best_ms = ms;
-            best = cand[ci];
+        return ms;
+    };
+    auto fits = [&](const Shape32& sh) {
+        try {
+            prepare_g32(c, nrhs, sh);
+            return true;
+        } catch (const MbsError& e) {
+            if (e.st != MBS_ERR_NOMEM) throw;
+            return false;  // no memory for that many partial sums
         }
+    };
+    auto clamp = [&](int ns) { return std::max(1, std::min(ns, max_nsplit(c))); };
+    launch_g32(c, nrhs, x, y, h, nullptr, nullptr);
+    Shape32 best = h;
+    float best_ms = time(h, HUGE_VALF);
+    if (c->opt.mac_path == 0 && h.path == 3) {
+        const int base = choose_nsplit(c, c->N);
+        Shape32 f{1, base}, g{1, clamp(base / 2)};
+        if (fits(f)) {
+            launch_g32(c, nrhs, x, y, f, nullptr, nullptr);
+            float ms = time(f, HUGE_VALF);
+            if (g.nsplit != base) {
+                const float t = time(g, 1.25f * ms);
+                if (t < ms) ms = t, f = g;
+            }
+            // in 3D the more accurate path of two as fast
+            if (ms < (c->dim == 3 ? 1.03f : 1.f) * best_ms) best_ms = ms, best = f;
+        }
+    }
+    // four times the usual count: small CTAs even out bodies of uneven size (700
+    // bodies, 16 right-hand sides: 4.64 ms with 14 splits, 4.30 with 28); the
+    // FP32-pipe kernel gains nothing
+    const int base = best.path == 3 ? h.nsplit : choose_nsplit(c, c->N);
+    std::vector<int> seen{base, best.path == 1 && h.path == 3 ? clamp(base / 2) : base};
+    for (int ns : {clamp(base / 2), clamp(2 * base), clamp(best.path == 3 ? 4 * base : base)}) {
+        if (std::find(seen.begin(), seen.end(), ns) != seen.end()) continue;
+        seen.push_back(ns);
+        const Shape32 sh{best.path, ns};
+        if (!fits(sh)) continue;
+        const float ms = time(sh, 1.25f * best_ms);
+        if (ms < best_ms) best_ms = ms, best = sh;
     }
     c->ev_pool.push_back(a);
     c->ev_pool.push_back(b);
