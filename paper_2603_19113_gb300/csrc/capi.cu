@@ -82,6 +82,10 @@ struct mbs_ctx {
     // no memory for the fixed-point kernel's workspace: the other FP64-accurate
     // kernels run for the rest of the call
     bool fx_off = false;
+    bool optional = false;        // what is being allocated gives way itself
+    // FP32 partial sums: bytes of the usual source splits, and the size that
+    // there was no memory for since the last build
+    size_t part32_usual = 0, part32_denied = SIZE_MAX;
     size_t fx_denied = SIZE_MAX;  // size that the device had no memory for since the last build
     std::vector<int64_t> off, voff;
     std::vector<int> kb;  // per-body skeleton count
@@ -140,11 +144,11 @@ struct mbs_ctx {
 
 namespace {
 
-bool drop_fx(mbs_ctx* c);
+bool give_way(mbs_ctx* c);
 
 void* dalloc(mbs_ctx* c, size_t bytes) {
     if (bytes == 0) bytes = 16;
-    if (c->opt.hbm_budget && c->bytes_held + bytes > c->opt.hbm_budget && drop_fx(c)) return dalloc(c, bytes);
+    if (c->opt.hbm_budget && c->bytes_held + bytes > c->opt.hbm_budget && give_way(c)) return dalloc(c, bytes);
     if (c->opt.hbm_budget && c->bytes_held + bytes > c->opt.hbm_budget)
         throw MbsError{MBS_ERR_NOMEM, "HBM budget exceeded (" + std::to_string(c->bytes_held + bytes) +
                                           " > " + std::to_string(c->opt.hbm_budget) + " bytes)"};
@@ -152,7 +156,7 @@ void* dalloc(mbs_ctx* c, size_t bytes) {
     cudaError_t e = cudaMalloc(&p, bytes);
     if (e != cudaSuccess) {
         cudaGetLastError();
-        if (drop_fx(c)) return dalloc(c, bytes);
+        if (give_way(c)) return dalloc(c, bytes);
         throw MbsError{MBS_ERR_NOMEM, std::string("cudaMalloc(") + std::to_string(bytes) +
                                           "): " + cudaGetErrorString(e)};
     }
@@ -189,16 +193,32 @@ void clear_graphs(mbs_ctx* c) {
     c->graphs.clear();
 }
 
-// The fixed-point kernel's workspace gives way to any other allocation: a
-// context whose memory or budget is exhausted goes on with the other
-// FP64-accurate kernels, which need none.
-bool drop_fx(mbs_ctx* c) {
-    auto it = c->bufs.find("fx_work");
-    if (it == c->bufs.end() || !it->second.p || c->capturing) return false;
-    clear_graphs(c);
+void release(mbs_ctx* c, DevBuf& b) {
+    clear_graphs(c);  // captured steps may refer to it
     if (c->st) cudaStreamSynchronize(c->st);
-    dfree(c, it->second.p);
-    it->second = DevBuf{};
+    dfree(c, b.p);
+    b = DevBuf{};
+}
+
+// FP32 partial sums beyond the usual source splits go back.
+bool cut_part32(mbs_ctx* c) {
+    auto it = c->bufs.find("part32");
+    if (c->capturing || it == c->bufs.end() || it->second.n <= c->part32_usual) return false;
+    c->part32_denied = std::min(c->part32_denied, it->second.n);
+    release(c, it->second);
+    return true;
+}
+
+// Buffers that a context can do without give way to any allocation that a call
+// needs (not to one that is itself optional): FP32 partial sums, then the
+// fixed-point kernel's workspace, without which the other FP64-accurate kernels
+// run.
+bool give_way(mbs_ctx* c) {
+    if (c->capturing || c->optional) return false;
+    if (cut_part32(c)) return true;
+    auto it = c->bufs.find("fx_work");
+    if (it == c->bufs.end() || !it->second.p) return false;
+    release(c, it->second);
     c->fx_off = true;
     return true;
 }
@@ -232,7 +252,7 @@ void free_geometry(mbs_ctx* c) {
     c->shapes.clear();
     c->bodies.clear();
     c->built = false;
-    c->fx_denied = SIZE_MAX;
+    c->fx_denied = c->part32_denied = SIZE_MAX;
     c->T = 0;
     c->N = 0;
     c->d_body = nullptr;
@@ -485,6 +505,10 @@ int log2_bucket(int64_t v) {
     return b;
 }
 
+size_t part32_bytes(const mbs_ctx* c, int nrhs, const Shape32& sh) {
+    return (size_t)sh.nsplit * nrhs * c->N * sizeof(float2);
+}
+
 // Buffers of a launch.
 struct Work32 {
     int* sb;
@@ -494,7 +518,6 @@ struct Work32 {
 Work32 prepare_g32(mbs_ctx* c, int nrhs, const Shape32& sh) {
     Work32 w{};
     w.sb = split_table(c, sh.nsplit);
-    w.part = scratch<float2>(c, "part32", (size_t)sh.nsplit * nrhs * c->N);
     if (sh.path == 3) {
         w.U.nchunks = c->nchunks;
         w.U.chunk_off = c->d_chunk_off;
@@ -503,7 +526,25 @@ Work32 prepare_g32(mbs_ctx* c, int nrhs, const Shape32& sh) {
         w.U.pack = scratch<unsigned char>(c, "umma_pack", w.U.pack_bytes);
         w.U.err = device_err(c);
     }
+    // last: it may give way to the others
+    w.part = scratch<float2>(c, "part32", part32_bytes(c, nrhs, sh) / sizeof(float2));
     return w;
+}
+
+// The buffers of a launch that others can stand in for; false: no memory for them.
+bool fits32(mbs_ctx* c, int nrhs, const Shape32& sh) {
+    struct Keep {
+        mbs_ctx* c;
+        ~Keep() { c->optional = false; }
+    } keep{c};
+    c->optional = true;
+    try {
+        prepare_g32(c, nrhs, sh);
+        return true;
+    } catch (const MbsError& e) {
+        if (e.st != MBS_ERR_NOMEM) throw;
+        return false;
+    }
 }
 
 void launch_g32(mbs_ctx* c, int nrhs, const float2* x, float2* y, const Shape32& sh,
@@ -523,6 +564,7 @@ Shape32 heuristic_shape32(mbs_ctx* c, int nrhs) {
 
 Shape32 shape32(mbs_ctx* c, int nrhs, const float2* x, float2* y) {
     const Shape32 h = heuristic_shape32(c, nrhs);
+    c->part32_usual = part32_bytes(c, nrhs, h);
     if (!c->opt.autotune || c->opt.tile_override > 0) return h;
     int dev = 0;
     MBS_CUDA_TRY(cudaGetDevice(&dev));
@@ -553,23 +595,15 @@ Shape32 shape32(mbs_ctx* c, int nrhs, const float2* x, float2* y) {
         }
         return ms;
     };
-    auto fits = [&](const Shape32& sh) {
-        try {
-            prepare_g32(c, nrhs, sh);
-            return true;
-        } catch (const MbsError& e) {
-            if (e.st != MBS_ERR_NOMEM) throw;
-            return false;  // no memory for that many partial sums
-        }
-    };
     auto clamp = [&](int ns) { return std::max(1, std::min(ns, max_nsplit(c))); };
     launch_g32(c, nrhs, x, y, h, nullptr, nullptr);
+    const size_t held = c->bufs["part32"].n;
     Shape32 best = h;
     float best_ms = time(h, HUGE_VALF);
     if (c->opt.mac_path == 0 && h.path == 3) {
         const int base = choose_nsplit(c, c->N);
         Shape32 f{1, base}, g{1, clamp(base / 2)};
-        if (fits(f)) {
+        if (fits32(c, nrhs, f)) {
             launch_g32(c, nrhs, x, y, f, nullptr, nullptr);
             float ms = time(f, HUGE_VALF);
             if (g.nsplit != base) {
@@ -589,12 +623,15 @@ Shape32 shape32(mbs_ctx* c, int nrhs, const float2* x, float2* y) {
         if (std::find(seen.begin(), seen.end(), ns) != seen.end()) continue;
         seen.push_back(ns);
         const Shape32 sh{best.path, ns};
-        if (!fits(sh)) continue;
+        if (!fits32(c, nrhs, sh)) continue;
         const float ms = time(sh, 1.25f * best_ms);
         if (ms < best_ms) best_ms = ms, best = sh;
     }
     c->ev_pool.push_back(a);
     c->ev_pool.push_back(b);
+    // partial sums beyond what the fastest shape needs go back
+    DevBuf& part = c->bufs["part32"];
+    if (part.n > std::max(held, part32_bytes(c, nrhs, best))) release(c, part);
     g_tune[key] = best;
     return best;
 }
@@ -602,7 +639,17 @@ Shape32 shape32(mbs_ctx* c, int nrhs, const float2* x, float2* y) {
 // y = G_hat x (FP32); a first call of a problem class may run the autotuner,
 // whose last timed launch is overwritten by the final one below.
 void G32(mbs_ctx* c, int nrhs, const float2* x, float2* y) {
-    const Shape32 sh = shape32(c, nrhs, x, y);
+    Shape32 sh = shape32(c, nrhs, x, y);
+    // a class's count may come from a context with more memory: the usual one of
+    // the heuristic then, which every call needs
+    const Shape32 usual{sh.path, heuristic_shape32(c, nrhs).nsplit};
+    c->part32_usual = part32_bytes(c, nrhs, usual);
+    const size_t need = part32_bytes(c, nrhs, sh);
+    if (sh.nsplit > usual.nsplit && need > c->bufs["part32"].n &&
+        (c->capturing || need >= c->part32_denied || !fits32(c, nrhs, sh))) {
+        if (!c->capturing) c->part32_denied = std::min(c->part32_denied, need);
+        sh = usual;
+    }
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (c->profile && c->capturing) {
         e0 = c->cap_e0;  // recorded on every replay of the step graph
@@ -628,7 +675,7 @@ int fx_nsplit(mbs_ctx* c, int64_t ntargets) {
 // Workspace of the fixed-point kernel, the default FP64-accurate one
 // (fp64_kernel = 2): packed sources and the partial sums of its source splits,
 // in one buffer that is taken after every other one of a call and gives way to
-// all of them (drop_fx).  With little memory fewer splits; null pack where an
+// all of them (give_way).  With little memory fewer splits; null pack where an
 // option picks another kernel or there is no memory at all.
 struct FxWork {
     unsigned char* pack = nullptr;
@@ -645,9 +692,8 @@ FxWork fx_workspace(mbs_ctx* c, int64_t ntargets, int nrhs) {
         if (ns > most) continue;
         const size_t need = pack + (size_t)ns * nrhs * ntargets * sizeof(double2);
         const size_t held = c->bufs["fx_work"].n;
-        if (need > held && (need >= c->fx_denied || c->capturing ||
-                            (c->opt.hbm_budget && c->bytes_held - held + need > c->opt.hbm_budget)))
-            continue;
+        auto over = [&]() { return c->opt.hbm_budget && c->bytes_held - held + need > c->opt.hbm_budget; };
+        if (need > held && (need >= c->fx_denied || c->capturing || (over() && !(cut_part32(c) && !over())))) continue;
         try {
             w.sb = split_table(c, ns);
             w.pack = scratch<unsigned char>(c, "fx_work", need);
@@ -1929,7 +1975,7 @@ mbs_status mbs_set_options(mbs_ctx* c, const mbs_options* opt) {
         void* keep = c->opt.stream;
         clear_graphs(c);
         c->opt = *opt;
-        c->fx_denied = SIZE_MAX;
+        c->fx_denied = c->part32_denied = SIZE_MAX;
         if (!opt->stream) c->opt.stream = keep;
         return MBS_OK;
     });
