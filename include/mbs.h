@@ -91,7 +91,9 @@ typedef struct mbs_options {
                             work only per body pair (3.4x faster than 0 on GB300 at N = 64,000, 8 RHS;
                             ~1e-13 relative instead of ~1e-16); 2 (default) automatic: 64-bit fixed point on
                             the integer multipliers, as accurate as 0 (9x faster than it at N = 15,000, 5 RHS).
-                            A context without memory for its workspace goes on with the other two: inside
+                            A context without memory for its workspace goes on with the other two, and so
+                            does a solve with a quarter of the body pairs at kappa r below about 16 (2D,
+                            32 bodies or more; then only where it is double-float): inside
                             solves double-float when 1e-14 ||S||_F (the FP64 residual floor it leaves, with
                             the root mean square of ||S_tau||_F over the bodies) is at most tol / 10, else
                             the FP64 pipe */

@@ -79,6 +79,7 @@ struct mbs_ctx {
     double snorm_rms = 0.0;  // root mean square over bodies of the Frobenius norm of S
     bool in_solve = false;
     bool df_active = false;
+    bool df_first = false;  // double-float even before the fixed-point kernel (solve_prefers_df)
     // no memory for the fixed-point kernel's workspace: the other FP64-accurate
     // kernels run for the rest of the call
     bool fx_off = false;
@@ -710,9 +711,36 @@ FxWork fx_workspace(mbs_ctx* c, int64_t ntargets, int nrhs) {
     return FxWork{};
 }
 
+// Whether the double-float kernel is the faster one, where a solve's tolerance
+// allows it: the fixed-point kernel sums body pairs outside its formats (2D:
+// kappa times their distance below about 16) on the FP64 pipe, the double-float
+// one only point pairs below kappa r = 4.  2D lattices, 8 right-hand sides,
+// share of such pairs, fixed point and double-float in ms: 40 bodies 0.24, 1.12
+// and 1.18; 0.71, 2.10 and 1.73; 160 bodies 0.08, 6.7 and 9.0; 0.28, 13.5 and
+// 11.6; 0.80, 33 and 20; 400 bodies 0.13, 44 and 56; 0.44, 110 and 78; but 10
+// bodies 1.0, 0.33 and 0.65 (the fixed-point kernel shares out few sources).
+bool solve_prefers_df(const mbs_ctx* c) {
+    if (c->T < 32) return false;
+    std::vector<double> centres((size_t)3 * c->T), rho(c->T);
+    for (int t = 0; t < c->T; ++t) {
+        for (int a = 0; a < 3; ++a) centres[3 * t + a] = c->bodies[t].c[a];
+        rho[t] = c->shapes[c->bodies[t].shape].bound_radius;
+    }
+    int64_t out = 0, all = 0;
+    for (int k = 0; k < 32; ++k) {  // targets spread over the bodies
+        const int64_t i = c->N * k / 32;
+        double x[3] = {0.0, 0.0, 0.0};
+        for (int a = 0; a < c->dim; ++a) x[a] = c->skel_world[(size_t)a * c->N + i];
+        const int own = (int)(std::upper_bound(c->off.begin(), c->off.end(), i) - c->off.begin()) - 1;
+        out += fx_outside(c->dim, c->kappa, x, own, c->T, centres.data(), rho.data());
+        all += c->T - 1;
+    }
+    return out > 0.25 * all;
+}
+
 void G64(mbs_ctx* c, int nrhs, const double2* x, double2* y) {
     // one body has no pairs: the kernel without a packing launch (45 us, not 60)
-    const FxWork fx = c->T > 1 ? fx_workspace(c, c->N, nrhs) : FxWork{};
+    const FxWork fx = c->T > 1 && !(c->in_solve && c->df_first) ? fx_workspace(c, c->N, nrhs) : FxWork{};
     const int ns = choose_nsplit(c, c->N);
     double2* part = nullptr;
     int* sb = nullptr;
@@ -2097,16 +2125,18 @@ mbs_status mbs_solve(mbs_ctx* c, int nrhs, const double* b, double* qhat, mbs_so
         if (nrhs < 1 || !b || !qhat) throw MbsError{MBS_ERR_ARG, "bad nrhs or null pointer"};
         const auto t0 = std::chrono::steady_clock::now();
         // FP64-accurate G_hat of this solve, should the fixed-point kernel be
-        // without memory under fp64_kernel = 2: double-float when the residual
+        // the slower one or without memory under fp64_kernel = 2: double-float when the residual
         // floor it leaves stays below a tenth of tol.  Its
         // ~1e-13 relative error in G_hat q reaches the residual through S:
         // measured, ~1e-14 relative per unit of ||S||; over many bodies the
         // errors add in norm, so the root mean square of ||S_tau||_F counts
         const int k64 = c->opt.fp64_kernel;
         const bool df = k64 == 1 || (k64 == 2 && 1e-14 * c->snorm_rms <= 0.1 * c->opt.tol);
-        if (k64 == 2 && df != c->df_active) {
+        const bool df_first = k64 == 2 && df && solve_prefers_df(c);
+        if (k64 == 2 && (df != c->df_active || df_first != c->df_first)) {
             clear_graphs(c);  // captured FP64 steps hold the other kernel
             c->df_active = df;
+            c->df_first = df_first;
         }
         struct InSolve {
             mbs_ctx* c;
@@ -2217,7 +2247,7 @@ mbs_status mbs_solve(mbs_ctx* c, int nrhs, const double* b, double* qhat, mbs_so
         finish_out(c, ox);
         inf.converged = conv ? 1 : 0;
         inf.rel_residual = relmax;
-        inf.fp64_kernel = k64 == 2 && !c->fx_off && c->T > 1 ? 2 : df ? 1 : 0;
+        inf.fp64_kernel = k64 == 2 && !df_first && !c->fx_off && c->T > 1 ? 2 : df ? 1 : 0;
         inf.seconds = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
         if (info) *info = inf;
         if (!conv) {

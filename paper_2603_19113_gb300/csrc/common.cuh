@@ -113,7 +113,8 @@ void launch_G_f64(const GLayout& L, double kappa, int nrhs, const double2* q, do
                   cudaEvent_t ev0 = nullptr, cudaEvent_t ev1 = nullptr);
 // FP64-accurate G_hat in double-float arithmetic on the FP32 pipe (gdf.cu);
 // d_centres: [T][3] body centres (FP64).  Selected by mbs_options.fp64_kernel = 1,
-// or by its default where a solve has no memory for the fixed-point kernel.
+// or by its default where a solve has no memory for the fixed-point kernel or
+// most pairs are outside its formats.
 // ev0/ev1 as for launch_G_f64: around the kernel passes, not the reduction.
 void launch_G_df(const GLayout& L, const double* d_centres, double kappa, int nrhs, const double2* q,
                  double2* y, double2* part, int nsplit, const int* d_split_body, cudaStream_t st,
@@ -134,6 +135,9 @@ size_t fx_pack_bytes(int dim, int64_t N, int T, int nrhs);
 FxPacked fx_packed(void* p, int dim, int64_t N, int T, int nrhs);
 int fx_groups(int64_t Nt, int T);
 int fx_tile(int64_t Nt, int T);
+// Bodies but `own` (centres [T][3], radii rho; host) that a target x is outside
+// the formats of.
+int fx_outside(int dim, double kappa, const double* x, int own, int T, const double* centres, const double* rho);
 void launch_G_fx(const GLayout& L, const double* d_centres, double kappa, int64_t Nt, const double* tgt,
                  const int* tbody, int nrhs, const double2* q, double2* y, double2* part, int nsplit,
                  const int* d_split_body, void* pack, cudaStream_t st, cudaEvent_t ev0 = nullptr,

@@ -14,7 +14,7 @@
 // the oracle's FP64 matvec (tests/test_gdf.py); on a GB300 the kernel agrees
 // with the FP64 kernel to 1.5e-13 (2D with and without the series fallback,
 // 3D).  Selected by mbs_options.fp64_kernel = 1, or by its default where a solve
-// has no memory for the fixed-point kernel (gfixed.cu).
+// has no memory for the fixed-point kernel (gfixed.cu) or many pairs outside its formats.
 #include "bessel.cuh"
 #include "common.cuh"
 #include "gdf_core.h"

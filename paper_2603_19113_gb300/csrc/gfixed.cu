@@ -348,4 +348,23 @@ int fx_groups(int64_t Nt, int T) {
     return tiles * std::min(T, 64) < 8LL * mbs_num_sms() ? 4 : 1;
 }
 
+int fx_outside(int dim, double kappa, const double* x, int own, int T, const double* centres, const double* rho) {
+    const FxKappa k = fx_kappa(dim, kappa);
+    int n = 0;
+    for (int t = 0; t < T; ++t) {
+        if (t == own) continue;
+        double D[3] = {0.0, 0.0, 0.0}, Dl[3] = {0.0, 0.0, 0.0}, R2 = 0.0, scale = 0.0;
+        for (int a = 0; a < dim; ++a) {
+            D[a] = x[a] - centres[3 * t + a];
+            R2 += D[a] * D[a];
+        }
+        FxBody<2> b2;
+        FxBody<3> b3;
+        const int es = fx_exponent(rho[t]);
+        n += dim == 2 ? !fx_body<2>(k, D, Dl, sqrt(R2), rho[t], es, b2, scale)
+                      : !fx_body<3>(k, D, Dl, sqrt(R2), rho[t], es, b3, scale);
+    }
+    return n;
+}
+
 int fx_tile(int64_t Nt, int T) { return FXT / fx_groups(Nt, T); }

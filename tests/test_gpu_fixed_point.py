@@ -236,3 +236,21 @@ def test_basis_update_teams(pkg, T, ks):
         ctx.set_options(precision=pkg.PREC_FP64)
         r = b - ctx.apply_operator(q)
         assert np.max(np.linalg.norm(r, axis=0) / np.linalg.norm(b, axis=0)) < 1e-11 * 1.01
+
+
+@pytest.mark.parametrize("T,kappa,kernel", [(160, 0.25, 1), (160, 40.0, 2), (12, 0.25, 2)])
+def test_kernel_of_a_low_frequency_solve(pkg, T, kappa, kernel):
+    """Double-float where the tolerance allows it and the formats leave out four in
+    five body pairs (160 bodies, kappa = 0.25: 20 ms a launch, fixed point 33)."""
+    wl = mi.config1(seed=0, T=T, kappa=kappa, nrhs=8)
+    with pkg.Context(2, kappa, precision=pkg.PREC_MIXED, tol=1e-9, restart=200) as ctx:
+        ctx.build_scattering_matrices(wl)
+        b = ctx.rhs(wl.boundary_data())
+        q, info = ctx.solve(b)
+        assert info["converged"] == 1 and info["fp64_kernel"] == kernel
+        ctx.set_options(precision=pkg.PREC_FP64, fp64_kernel=0)
+        r = b - ctx.apply_operator(q)
+        assert np.max(np.linalg.norm(r, axis=0) / np.linalg.norm(b, axis=0)) < 1e-9 * 1.01
+        if kernel == 1:  # a tolerance that double-float does not reach
+            ctx.set_options(precision=pkg.PREC_MIXED, fp64_kernel=2, tol=1e-13, max_iter=3)
+            assert ctx.solve(b, raise_on_noconv=False)[1]["fp64_kernel"] == 2
