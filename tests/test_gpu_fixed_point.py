@@ -254,3 +254,28 @@ def test_kernel_of_a_low_frequency_solve(pkg, T, kappa, kernel):
         if kernel == 1:  # a tolerance that double-float does not reach
             ctx.set_options(precision=pkg.PREC_MIXED, fp64_kernel=2, tol=1e-13, max_iter=3)
             assert ctx.solve(b, raise_on_noconv=False)[1]["fp64_kernel"] == 2
+
+
+@pytest.mark.parametrize("case", ["2d", "2d_high", "2d_low", "3d", "3d_low"])
+@pytest.mark.parametrize("nrhs", [1, 8])
+def test_fixed_point_accuracy(pkg, case, nrhs):
+    """Sampled rows against 30-digit sums over the same coordinates.  A pair is off
+    by 1e-15 in phi and its product, by kappa 2^-53 through the rounding of a source's
+    offset (radius 1) and by kappa 2^e 2^-58 <= kappa 2^-54 in the phase, pairs of
+    different sources independently: five times the root of the sum of their squares."""
+    mp = pytest.importorskip("mpmath")
+    mp.mp.dps = 30
+    wl = mi.tiny_3d(seed=0, T=5, kappa=0.5, nth=10, nph=14, p=141, k=70) if case == "3d_low" else _WL[case]()
+    ctx, x, body, off = _ctx(pkg, wl)
+    q = _rand((ctx.N, nrhs), 4)
+    y = ctx.apply_G(q)
+    for i in np.linspace(0, ctx.N - 1, 5).astype(int):
+        phi = []
+        for j in range(ctx.N):
+            r = mp.sqrt(sum((mp.mpf(float(a)) - mp.mpf(float(b))) ** 2 for a, b in zip(x[i], x[j])))
+            phi.append(mp.mpc(0) if body[i] == body[j] else mp.mpc(0, 0.25) * mp.hankel1(0, wl.kappa * r) if wl.dim == 2 else
+                       mp.exp(mp.mpc(0, wl.kappa) * r) / (4 * mp.pi * r))
+        for c in range(nrhs):
+            ref = mp.fsum(p * mp.mpc(complex(v)) for p, v in zip(phi, q[:, c]))
+            size = float(mp.sqrt(mp.fsum(abs(p) ** 2 * abs(v) ** 2 for p, v in zip(phi, q[:, c].tolist()))))
+            assert abs(mp.mpc(complex(y[i, c])) - ref) < 5 * size * (1e-15 + wl.kappa * (2.0 ** -53 + 2.0 ** -54))

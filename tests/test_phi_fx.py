@@ -98,3 +98,29 @@ def test_bodies_outside_the_formats_are_refused(lib):
         out, ok, raw = np.zeros((1, 2)), np.ones(1, np.int32), np.zeros((1, 2), np.int64)
         lib.phi_fx_batch(dim, ctypes.c_double(kappa), 1, _p(D), _p(r), _p(es), _p(dj), _p(out), _p(ok), _p(raw))
         assert ok[0] == 0, (dim, kappa, D)
+
+
+@pytest.mark.parametrize("kappa,hi", [(0.01, 50), (1.0, 8)])
+def test_phi_near_bodies_at_low_frequency(lib, kappa, hi):
+    """3D, where the phase carries no error and the modulus all of it.  The result
+    is rounded to FP64 twice (2.2e-16 together), its scale once (1.1e-16), and the
+    integers end at 2^-56 of the nearest point's amplitude or 2^-54 of the farthest's
+    (5.6e-17): 4e-16, which plain FP64 does not stay below."""
+    mp.mp.dps = 40
+    rng = np.random.default_rng(5)
+    n = 1500
+    rho = rng.uniform(0.55, 1.1, n)
+    R = rho * np.exp(rng.uniform(np.log(1.3), np.log(hi), n))
+    u, w = rng.normal(size=(n, 3)), rng.normal(size=(n, 3))
+    D = np.ascontiguousarray(R[:, None] * u / np.linalg.norm(u, axis=1)[:, None])
+    delta = w / np.linalg.norm(w, axis=1)[:, None] * (rho * rng.uniform(0, 1, n))[:, None]
+    es = np.array([int(np.frexp(r * (1 + 1e-6))[1]) for r in rho], np.int32)
+    dj = np.array([[int(np.rint(d * 2.0 ** (63 - e))) for d in row] for row, e in zip(delta, es)], dtype=np.int64)
+    out, ok, raw = np.zeros((n, 2)), np.zeros(n, np.int32), np.zeros((n, 2), np.int64)
+    lib.phi_fx_batch(3, ctypes.c_double(kappa), n, _p(D), _p(rho), _p(es), _p(dj), _p(out), _p(ok), _p(raw))
+    assert (ok == 1).sum() > n // 2
+    for i in np.nonzero(ok == 1)[0]:
+        r = mp.sqrt(sum((mp.mpf(float(D[i, a])) - mp.mpf(int(dj[i, a])) / mp.mpf(2) ** (63 - int(es[i]))) ** 2 for a in range(3)))
+        ref = mp.exp(mp.mpc(0, 1) * kappa * r) / (4 * mp.pi * r)
+        err = float(abs(mp.mpc(float(out[i, 0]), float(out[i, 1])) - ref) / abs(ref))
+        assert err < 4e-16 + kappa * 2.0 ** (np.ceil(np.log2((R[i] + rho[i]) * 1.0001)) - 58), i
