@@ -173,7 +173,7 @@ constexpr double FX_RMIN = 0.0626;  // least r / 2^e
 template <int DIM>
 FX_HD bool fx_body(const FxKappa& k, const double* D, const double* Dl, double R, double rho, int es, FxBody<DIM>& b, double& scale) {
     const double rmax = (R + rho) * (1.0 + 1e-6);
-    if (!(rmax > 1e-90 && rmax < 1e90)) return false;
+    if (!(rmax > 1e-17 && rmax < 1e18)) return false;  // R comes from FP32 squares, R > rho: normal numbers
     int e = fx_exponent(rmax);
     if (e < es) e = es;
     const double rmin = (R - rho) * (1.0 - 1e-6);

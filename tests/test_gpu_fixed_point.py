@@ -279,3 +279,23 @@ def test_fixed_point_accuracy(pkg, case, nrhs):
             ref = mp.fsum(p * mp.mpc(complex(v)) for p, v in zip(phi, q[:, c]))
             size = float(mp.sqrt(mp.fsum(abs(p) ** 2 * abs(v) ** 2 for p, v in zip(phi, q[:, c].tolist()))))
             assert abs(mp.mpc(complex(y[i, c])) - ref) < 5 * size * (1e-15 + wl.kappa * (2.0 ** -53 + 2.0 ** -54))
+
+
+def _scaled(wl, s):
+    import dataclasses
+    shapes = [dataclasses.replace(h, x=h.x * s, y=h.y * s, z=h.z * s, proxy_radius=h.proxy_radius * s,
+                                  bound_radius=h.bound_radius * s) for h in wl.shapes]
+    return dataclasses.replace(wl, kappa=wl.kappa / s, shapes=shapes, centres=wl.centres * s)
+
+
+@pytest.mark.parametrize("e", [-75, -70, -62, 62, 70])
+def test_sums_in_any_unit_of_length(pkg, e):
+    """2D sums depend on kappa times lengths alone: the FP64-accurate ones of a
+    geometry 2^e times as large, where squares leave FP32's range too."""
+    wl = _WL["2d"]()
+    ctx, x, body, _ = _ctx(pkg, wl)
+    big, xb, _, _ = _ctx(pkg, _scaled(wl, 2.0 ** e))
+    if not np.array_equal(xb, x * 2.0 ** e):
+        pytest.skip("another skeleton")
+    q = _rand((ctx.N, 3), 1)
+    assert _rel(big.apply_G(q), ctx.apply_G(q)) < 1e-12

@@ -124,3 +124,16 @@ def test_phi_near_bodies_at_low_frequency(lib, kappa, hi):
         ref = mp.exp(mp.mpc(0, 1) * kappa * r) / (4 * mp.pi * r)
         err = float(abs(mp.mpc(float(out[i, 0]), float(out[i, 1])) - ref) / abs(ref))
         assert err < 4e-16 + kappa * 2.0 ** (np.ceil(np.log2((R[i] + rho[i]) * 1.0001)) - 58), i
+
+
+@pytest.mark.parametrize("dim", [2, 3])
+@pytest.mark.parametrize("size", [1e-25, 1e-20, 1e-16, 1e17, 1e20])
+def test_bodies_whose_squared_distance_leaves_fp32_are_refused(lib, dim, size):
+    """|D| is a root of FP32 squares: below 1e-19 they have lost their digits, above
+    1e19 they overflow.  Bodies of any size between keep the formats."""
+    kappa, D, r = 30.0 / size, np.zeros((1, dim)), np.array([size])
+    D[0, 0] = 4.0 * size
+    es, dj = np.array([int(np.frexp(size * (1 + 1e-6))[1])], np.int32), np.zeros((1, dim), np.int64)
+    out, ok, raw = np.zeros((1, 2)), np.ones(1, np.int32), np.zeros((1, 2), np.int64)
+    lib.phi_fx_batch(dim, ctypes.c_double(kappa), 1, _p(D), _p(r), _p(es), _p(dj), _p(out), _p(ok), _p(raw))
+    assert ok[0] == (1 if 1e-17 < size < 1e18 else 0)
