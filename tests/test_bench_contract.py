@@ -52,3 +52,18 @@ def test_reference_arm_under_torchrun_prints_once():
     lines = _json_lines(p.stdout)
     assert len(lines) == 1
     _check_line(lines[0], 2)
+
+
+def test_side_measurements_follow_short_runs_only(monkeypatch):
+    """A run of many steps prints its line without the plain FP64 solve and the
+    serving traces; the default run has them."""
+    sys.path.insert(0, ROOT)
+    import bench
+    monkeypatch.setattr(sys, "argv", ["bench.py"])
+    assert bench.sides(bench.parse(), 5 * 14.0) == (True, True)
+    monkeypatch.setattr(sys, "argv", ["bench.py", "--steps", "20", "--warmup", "5"])
+    assert bench.sides(bench.parse(), 25 * 14.0) == (False, False)
+    monkeypatch.setattr(sys, "argv", ["bench.py", "--no-fp64", "--side-after", "1000"])
+    assert bench.sides(bench.parse(), 25 * 14.0) == (False, True)
+    monkeypatch.setattr(sys, "argv", ["bench.py", "--config", "2"])
+    assert bench.sides(bench.parse(), 1.0) == (False, False)
