@@ -299,3 +299,31 @@ def test_sums_in_any_unit_of_length(pkg, e):
         pytest.skip("another skeleton")
     q = _rand((ctx.N, 3), 1)
     assert _rel(big.apply_G(q), ctx.apply_G(q)) < 1e-12
+
+
+@pytest.mark.parametrize("T,nrhs,ks,m_per_k", [
+    (160, 3, (24, 37, 64), 2),   # 2 right-hand sides a CTA would take 320 CTAs: 3 a CTA
+    (50, 6, (24, 37, 64), 2),    # 2 a CTA
+    (40, 7, (24, 37, 64), 2),    # 4 a CTA, the last 3
+    (160, 11, (24, 37, 64), 2),  # 8 a CTA, the last 3; one column alone: the general kernel
+    (80, 8, (24, 37, 65), 2),    # 130 points: 8 row groups
+    (64, 11, (24, 37, 51), 5),   # 255 points
+    (64, 11, (24, 48, 64), 4),   # 256 points
+])
+def test_blocked_rhs_and_reconstruction(pkg, T, nrhs, ks, m_per_k):
+    """Several right-hand sides a CTA (152 SMs) give each column what it gets alone,
+    where it takes another kernel or another share of a CTA: to the bit."""
+    wl = mi.tiny_2d(seed=5, T=T, kappa=15.0, nrhs=nrhs, ks=ks, m_per_k=m_per_k)
+    with pkg.Context(2, wl.kappa) as ctx:
+        ctx.build_scattering_matrices(wl)
+        v, q = wl.boundary_data(), _rand((ctx.N, nrhs), 3)
+        b, qm = ctx.rhs(v), ctx.reconstruct(v, q)
+        for r in range(nrhs):
+            assert np.array_equal(ctx.rhs(v[:, r]), b[:, r])
+            assert np.array_equal(ctx.reconstruct(v[:, r], q[:, r]), qm[:, r])
+
+
+def test_fixed_point_sums_at_full_size(pkg):
+    """The bench workload's 256 sampled rows through the default kernel."""
+    from test_gpu_parity import test_G_full_size_config1_sampled_rows as full_size
+    full_size(pkg, 0, 2)
