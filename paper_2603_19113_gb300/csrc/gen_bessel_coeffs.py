@@ -6,7 +6,8 @@ both smooth functions of t = xa / x in (0, 1] tending to f = 1, g = 0 as
 x -> infinity (Hankel's asymptotic form, DLMF 10.17.1 / 10.18).  Each is fitted
 by a Chebyshev series in u = 2 t - 1 on [-1, 1] from high-precision values of
 J0 and Y0 (mpmath), and written out as monomial coefficients in u, highest
-degree first, for Horner evaluation.
+degree first, for Horner evaluation.  The fixed-point kernel's fits for x >= 64
+(fx_fit) are of what Hankel's leading terms leave.
 
 Run:  python gen_bessel_coeffs.py > bessel_coeffs.h
 """
@@ -56,6 +57,21 @@ def fit(xa, deg, nodes=160):
     return cf[::-1], cg[::-1], ef, eg
 
 
+def fx_fit():
+    """F and G of f = 1 - v/16 + v^2 F(v) and g = -s/8 + s v G(v), s = 1/x and
+    v = s^2 <= 2^-12: interpolated at three Chebyshev points, lowest degree first."""
+    top, n = mp.mpf(2) ** -12, 3
+    at = [top / 2 * (1 + mp.cos(mp.pi * (2 * i + 1) / (2 * n))) for i in range(n)]
+    F, G = [], []
+    for v in at:
+        s = mp.sqrt(v)
+        h = mp.hankel1(0, 1 / s) * mp.sqrt(mp.pi / (2 * s)) * mp.exp(-1j * (1 / s - mp.pi / 4))
+        F.append((abs(h) - 1 + v / 16) / v ** 2)
+        G.append((mp.arg(h) + s / 8) / (s * v))
+    A = mp.matrix([[v ** j for j in range(n)] for v in at])
+    return [[float(c) for c in mp.lu_solve(A, mp.matrix(y))] for y in (F, G)]
+
+
 def main(out=sys.stdout):
     out.write("// Generated by gen_bessel_coeffs.py: modulus/phase fits of H0^(1).\n")
     out.write("// f(x) = |H0(x)| sqrt(pi x / 2), g(x) = arg H0(x) - (x - pi/4), for x >= XA,\n")
@@ -72,6 +88,10 @@ def main(out=sys.stdout):
             body = ", ".join(f"{c:.17e}{suf}" for c in cc)
             out.write(f"#define MBS_{name}_{lab} {{{body}}}\n")
         out.write("\n")
+    out.write("// FX_X64: x >= 64, degree 2 in 1 / x^2, lowest degree first: what Hankel's leading terms leave\n")
+    for lab, cc in zip("FG", fx_fit()):
+        out.write(f"#define MBS_FX_X64_{lab} {{{', '.join(f'{c:.17e}' for c in cc)}}}\n")
+    out.write("\n")
 
 
 if __name__ == "__main__":

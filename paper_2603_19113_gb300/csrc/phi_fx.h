@@ -244,12 +244,13 @@ FX_CONST FxTab<MBS_F64_X4_DEG + 1> c_fx4G = fx_table(kFx4G, FX_INV2PI, 0.0);
 // kappa r >= 64: with s = 1 / x, v = s^2, f = 1 - v/16 + v^2 F(v) and
 // g = -s/8 + s v G(v) (Hankel's expansion, leading terms exact, F and G fitted
 // on v <= 2^-12; errors 3e-18 and 4e-17)
-constexpr unsigned FX_F0 = (unsigned)(0.10351562495188254706 * 0x1p34 + 0.5);
-constexpr unsigned FX_F1 = (unsigned)(0.54284313075330579387 * 0x1p23 + 0.5);
-constexpr unsigned FX_F2 = (unsigned)(5.8098521221942328077 * 0x1p12 + 0.5);
-constexpr unsigned FX_G0 = (unsigned)(0.065104166656079809861 * FX_INV2PI * 0x1p37 + 0.5);
-constexpr unsigned FX_G1 = (unsigned)(0.20956953171157405515 * FX_INV2PI * 0x1p26 + 0.5);
-constexpr unsigned FX_G2 = (unsigned)(1.6295224694592193371 * FX_INV2PI * 0x1p15 + 0.5);
+constexpr double kFx64F[] = MBS_FX_X64_F, kFx64G[] = MBS_FX_X64_G;  // signs alternate
+constexpr unsigned FX_F0 = (unsigned)(kFx64F[0] * 0x1p34 + 0.5);
+constexpr unsigned FX_F1 = (unsigned)(-kFx64F[1] * 0x1p23 + 0.5);
+constexpr unsigned FX_F2 = (unsigned)(kFx64F[2] * 0x1p12 + 0.5);
+constexpr unsigned FX_G0 = (unsigned)(kFx64G[0] * FX_INV2PI * 0x1p37 + 0.5);
+constexpr unsigned FX_G1 = (unsigned)(-kFx64G[1] * FX_INV2PI * 0x1p26 + 0.5);
+constexpr unsigned FX_G2 = (unsigned)(kFx64G[2] * FX_INV2PI * 0x1p15 + 0.5);
 
 // e^{2 pi i theta} at 2^62, theta in turns at 2^64: the nearest of 1024 steps,
 // times cos t + i sin t of the rest |t| <= pi / 1024

@@ -137,3 +137,19 @@ def test_bodies_whose_squared_distance_leaves_fp32_are_refused(lib, dim, size):
     out, ok, raw = np.zeros((1, 2)), np.ones(1, np.int32), np.zeros((1, 2), np.int64)
     lib.phi_fx_batch(dim, ctypes.c_double(kappa), 1, _p(D), _p(r), _p(es), _p(dj), _p(out), _p(ok), _p(raw))
     assert ok[0] == (1 if 1e-17 < size < 1e18 else 0)
+
+
+def test_fits_are_the_generators():
+    """The coefficients for kappa r >= 64 are what their generator gives."""
+    import re
+    import sys
+    csrc = os.path.join(ROOT, "paper_2603_19113_gb300", "csrc")
+    sys.path.insert(0, csrc)
+    try:
+        import gen_bessel_coeffs as gen
+    finally:
+        sys.path.remove(csrc)
+    text = open(os.path.join(csrc, "bessel_coeffs.h")).read()
+    for lab, want in zip("FG", gen.fx_fit()):
+        got = re.search(r"MBS_FX_X64_%s \{(.*)\}" % lab, text).group(1)
+        assert [float(c) for c in got.split(",")] == want
