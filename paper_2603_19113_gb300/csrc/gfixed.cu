@@ -3,15 +3,17 @@
 // y_i = sum over the skeleton sources j of other bodies of phi(t_i - x_j) q_j,
 // for FP64 operators, refinement residuals and field evaluation.
 //
-// phi comes from phi_fx.h (72 wide integer multiply-adds a pair in 2D, against
+// phi comes from phi_fx.h (73 wide integer multiply-adds a pair in 2D, against
 // about 50 FP64 operations that take 16 times as long each); the product with
 // the right-hand sides, integers of 60 bits relative to the largest |q| of a
-// source body, takes 4 wide multiply-adds and 8 FP32 ones (the cross terms of
-// high and low words, whose 24 bits end near 2^-56) a pair and right-hand side,
-// and goes into FP64 sums once per 64 sources.  237 bodies of 64
-// points, 5 right-hand sides: 4.35 ms, 42 ms on the FP64 pipe; 1000 bodies and
+// source body, takes 4 wide multiply-adds and 8 FP32 ones a pair and right-hand
+// side, and goes into FP64 sums once per 64 sources.  The FP32 ones are the cross
+// terms of high words (27 bits of phi, 28 of q) and low ones, 2^-28 of a product
+// of the largest entries: their 24 bits end near 2^-52 of it, up to 8 times
+// coarser in a sum of 16.  237 bodies of 64
+// points, 5 right-hand sides: 4.40 ms, 42 ms on the FP64 pipe; 1000 bodies and
 // 4096 targets, 8 right-hand sides: 5.7 ms and 53.6 ms.  The wide multiply-adds
-// alone, 32 a clock and SM, would take 2.1 ms of the 4.35; issue slots are 57 %
+// alone, 32 a clock and SM, would take 2.1 ms of the 4.40; issue slots are 57 %
 // busy, the ALU 52 %, and warps wait for dispatch, busy pipes and dependent
 // results in about equal parts.
 //

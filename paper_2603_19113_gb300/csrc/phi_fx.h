@@ -37,8 +37,8 @@ struct fx2 {
 FX_HD int fx_hi(fx_i64 a) { return (int)(a >> 32); }
 FX_HD unsigned fx_hiu(fx_u64 a) { return (unsigned)(a >> 32); }
 // a b + c and the high half of a b.  On the device as explicit wide
-// multiply-adds (one instruction at 62 a clock and SM): from 64-bit C
-// expressions the compiler makes three, and the 32-bit high product is two.
+// multiply-adds (32 a clock and SM), whatever a compiler makes of 64-bit
+// expressions.
 FX_HD fx_i64 fx_madw(int a, int b, fx_i64 c) {
 #if defined(__CUDA_ARCH__)
     fx_i64 d;
@@ -163,8 +163,9 @@ struct FxBody {
 };
 
 // Lengths below 2^-4 of 2^e would leave the integer formats: such bodies
-// (targets within about a fifteenth of the body's radius of its hull) and the
-// ranges below go to the FP64 evaluation instead.
+// (2^e is 2 to 4 times the radius there, so targets within an eighth to a quarter
+// of the radius of the hull) and the ranges below go to the FP64 evaluation
+// instead.
 constexpr double FX_RMIN = 0.0626;  // least r / 2^e
 
 // Constants of a body at offset D + Dl from the target (|D| = R), radius rho, with

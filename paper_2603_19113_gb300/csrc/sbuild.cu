@@ -967,9 +967,8 @@ __global__ void __launch_bounds__(256) recon_kernel(const RhsBody* __restrict__ 
 constexpr int RB = 8;          // right-hand sides per CTA = warps
 constexpr int RB_GROUPS = 8;   // groups of 32 rows: m <= 256
 
-// Sum over the warp of each of the 2 G values, by the tree lane ^ 16, 8, 4, 2, 1;
-// lane 4 i + (0..3) ends with the sum of value i (i < 8; G = 4) or 2 i + ... (see
-// rows_total).
+// One step of the tree lane ^ 16, 8, 4, 2, 1 for a value that this lane keeps: the
+// partner's copy of it is added.
 __device__ __forceinline__ double xchg_add(double keep, double send, int o) {
     return keep + __shfl_xor_sync(0xffffffffu, send, o);
 }
