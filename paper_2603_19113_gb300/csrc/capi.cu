@@ -283,13 +283,20 @@ bool is_device_ptr(const void* p) {
     return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
+// Work on the legacy default stream and the capture of a stream that
+// synchronises with it (a caller's) exclude each other.
+std::mutex g_legacy_mu;
+
 // The context's work from here on follows what the legacy default stream holds:
 // device arguments may still be in the making there, and the context's own
 // stream, which does not wait for it by itself, is not known to the caller.
 void after_default_stream(mbs_ctx* c) {
     if (c->ordered) return;
     if (!c->caller) MBS_CUDA_TRY(cudaEventCreateWithFlags(&c->caller, cudaEventDisableTiming));
-    MBS_CUDA_TRY(cudaEventRecord(c->caller, cudaStreamLegacy));
+    {
+        std::lock_guard<std::mutex> lk(g_legacy_mu);
+        MBS_CUDA_TRY(cudaEventRecord(c->caller, cudaStreamLegacy));
+    }
     MBS_CUDA_TRY(cudaStreamWaitEvent(c->st, c->caller, 0));
     c->ordered = true;
 }
@@ -1112,6 +1119,9 @@ StepGraph* run_step_graph(mbs_ctx* c, const std::array<int64_t, 8>& key, int pre
             c->graphs_off = true;
             return nullptr;
         };
+        unsigned flags = cudaStreamNonBlocking;
+        std::unique_lock<std::mutex> lk(g_legacy_mu, std::defer_lock);
+        if (!c->own_stream && cudaStreamGetFlags(c->st, &flags) == cudaSuccess && !(flags & cudaStreamNonBlocking)) lk.lock();
         if (cudaStreamBeginCapture(c->st, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return fail();
         c->capturing = true;
         c->cap_e0 = g.e0;
@@ -1125,6 +1135,7 @@ StepGraph* run_step_graph(mbs_ctx* c, const std::array<int64_t, 8>& key, int pre
         }
         cudaGraph_t graph = nullptr;
         const cudaError_t ee = cudaStreamEndCapture(c->st, &graph);
+        if (lk.owns_lock()) lk.unlock();
         c->capturing = false;
         g.launches = g_mbs_launches.load() - l0;
         g_mbs_launches.fetch_sub(g.launches);  // nothing ran during the capture

@@ -55,3 +55,41 @@ def test_arguments_in_the_making(pkg, maker, runner):
                 got = f(*late)
             torch.cuda.synchronize()
             assert np.array_equal(got.cpu().numpy(), want)
+
+
+def test_beside_a_context_that_captures_on_a_blocking_stream(pkg):
+    """One thread solves on a stream of the kind that the default stream waits for,
+    its steps captured as graphs; another passes device arguments all the while."""
+    import ctypes
+    import threading
+    import torch
+    wl = mi.tiny_2d(seed=1, T=9, kappa=6.0, nrhs=3)
+    rt = ctypes.CDLL("libcudart.so.13")
+    st = ctypes.c_void_p()
+    assert rt.cudaStreamCreate(ctypes.byref(st)) == 0
+    failed, done = [], threading.Event()
+    with pkg.Context(2, wl.kappa, stream=st.value, restart=30, tol=1e-10) as a, pkg.Context(2, wl.kappa) as b:
+        a.build_scattering_matrices(wl)
+        b.build_scattering_matrices(wl)
+        rhs = a.rhs(wl.boundary_data())
+        q = torch.from_numpy(np.ascontiguousarray(rhs.T)).cuda().T
+        want = b.apply_G(rhs)
+
+        def solve():
+            try:
+                for _ in range(20):
+                    a.set_options(tol=1e-10)  # drops the captured steps
+                    a.solve(rhs, raise_on_noconv=False)
+            except Exception as e:
+                failed.append(e)
+            done.set()
+
+        t = threading.Thread(target=solve)
+        t.start()
+        got = []
+        while not done.is_set():  # no torch work in between: its default stream minds captures too
+            got.append(b.apply_G(q))
+        t.join()
+        assert not failed and len(got) > 20
+        assert all(np.array_equal(y.cpu().numpy(), want) for y in got)
+    assert rt.cudaStreamDestroy(st) == 0
