@@ -90,13 +90,13 @@ typedef struct mbs_options {
                             0 on the FP64 pipe; 1 G_hat in double-float arithmetic on the FP32 pipe, with FP64
                             work only per body pair (3.4x faster than 0 on GB300 at N = 64,000, 8 RHS;
                             ~1e-13 relative instead of ~1e-16); 2 (default) automatic: 64-bit fixed point on
-                            the integer multipliers, as accurate as 0 (9x faster than it at N = 15,000, 5 RHS).
-                            A context without memory for its workspace goes on with the other two, and so
-                            does a solve with a quarter of the body pairs at kappa r below about 16 (2D,
-                            32 bodies or more; then only where it is double-float): inside
-                            solves double-float when 1e-14 ||S||_F (the FP64 residual floor it leaves, with
-                            the root mean square of ||S_tau||_F over the bodies) is at most tol / 10, else
-                            the FP64 pipe */
+                            the integer multipliers, as accurate as 0 (9x faster than it at N = 15,000, 5 RHS;
+                            entries of q count 60 bits below the largest of their body and column).
+                            Inside solves double-float is allowed when 1e-14 ||S||_F (the FP64 residual
+                            floor it leaves, with the root mean square of ||S_tau||_F over the bodies) is at
+                            most tol / 10, and then taken where a quarter of the pairs of 32 bodies or more
+                            lie below kappa r of about 16 (2D).  A call without memory for the fixed-point
+                            workspace goes on with double-float where allowed, else the FP64 pipe */
     int sbuild_threads;  /* threads per CTA of the S build (128, 256 or 512); 0 (default): 256 (the build
                             is FP64-pipe-bound: the three sizes measured within 2 % on GB300); -1: tuned on the
                             first build of a size class (when autotune is on), at the cost of ~half a build */
