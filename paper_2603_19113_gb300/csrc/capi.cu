@@ -145,6 +145,14 @@ struct mbs_ctx {
 
 namespace {
 
+// Host arrays that queued copies read or write stay until the copies are done:
+// declared after them, this waits for the stream before they go, on errors too.
+// (Beyond 64 KB the device may read pageable memory after the call has returned.)
+struct Drain {
+    cudaStream_t st;
+    ~Drain() { cudaStreamSynchronize(st); }
+};
+
 bool give_way(mbs_ctx* c);
 
 void* dalloc(mbs_ctx* c, size_t bytes) {
@@ -1003,6 +1011,7 @@ GmresStats gmres(mbs_ctx* c, int nrhs, const V* b, V* x, bool x_zero, double tol
             }
             for (int i = 0; i < mq; ++i) y[(size_t)i * nrhs + q] = make_double2(yq[i].real(), yq[i].imag());
         }
+        const Drain drain{c->st};
         if (jdone > 0) {
             MBS_CUDA_TRY(cudaMemcpyAsync(d_h, y.data(), y.size() * sizeof(double2),
                                          cudaMemcpyHostToDevice, c->st));
@@ -1344,6 +1353,7 @@ GmresStats bgmres(mbs_ctx* c, int s, const V* b, V* x, bool x_zero, double tol, 
         if (Mj > 0) {
             double2* d_y = scratch<double2>(c, "bg_y", (size_t)restart * s * s);
             std::vector<double2> stage;
+            const Drain drain{c->st};
             from_host_cd(Y, d_y, c->st, stage);
             launch_ts_update<V>(basis, Mj, d_y, 1.0, x, s, N, c->st, d_coef, device_err(c));
         }
@@ -1421,9 +1431,11 @@ mbs_status guarded(mbs_ctx* c, F&& f) {
         if (s == MBS_OK) c->err.clear();
         return s;
     } catch (const MbsError& e) {
+        if (c->st) cudaStreamSynchronize(c->st);  // the caller's arrays may still be in use
         c->err = e.msg;
         return e.st;
     } catch (const std::exception& e) {
+        if (c->st) cudaStreamSynchronize(c->st);
         c->err = e.what();
         return MBS_ERR_CUDA;
     }
@@ -1570,6 +1582,7 @@ void setup_layout(mbs_ctx* c) {
     c->d_centres = galloc<double>(c, (size_t)5 * T);
     c->d_pair = galloc<float4>(c, (size_t)T * T);
     c->d_pair_phi0 = d == 3 ? galloc<float>(c, (size_t)T * T) : nullptr;
+    const Drain points{c->st};
     MBS_CUDA_TRY(cudaMemcpyAsync(c->d_body, body.data(), N * sizeof(int), cudaMemcpyHostToDevice, c->st));
     MBS_CUDA_TRY(cudaMemcpyAsync(c->d_off, c->off.data(), (T + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, c->st));
     MBS_CUDA_TRY(cudaMemcpyAsync(c->d_loc32, loc32.data(), loc32.size() * sizeof(float), cudaMemcpyHostToDevice, c->st));
@@ -1587,6 +1600,7 @@ void setup_layout(mbs_ctx* c) {
         for (int k = 0; k < nc; ++k) chunk_body.push_back(t);
     }
     c->nchunks = chunk_off[T];
+    const Drain chunks{c->st};
     c->d_chunk_off = galloc<int>(c, T + 1);
     c->d_chunk_body = galloc<int>(c, std::max<size_t>(1, chunk_body.size()));
     MBS_CUDA_TRY(cudaMemcpyAsync(c->d_chunk_off, chunk_off.data(), (T + 1) * sizeof(int),
@@ -1631,6 +1645,7 @@ void setup_layout(mbs_ctx* c) {
         for (int a = 0; a < 3; ++a) mb[t].c[a] = c->bodies[t].c[a];
         for (int a = 0; a < 9; ++a) mb[t].R[a] = c->bodies[t].R[a];
     }
+    const Drain tables{c->st};
     c->d_mfsb = galloc<MfsBody>(c, T);
     MBS_CUDA_TRY(cudaMemcpyAsync(c->d_mfsb, mb.data(), T * sizeof(MfsBody), cudaMemcpyHostToDevice, c->st));
     MBS_CUDA_TRY(cudaMemcpyAsync(c->d_k, c->kb.data(), T * sizeof(int), cudaMemcpyHostToDevice, c->st));

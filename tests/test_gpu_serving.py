@@ -136,3 +136,25 @@ def test_shortest_work_first_admission(pkg):
     start = [srv.poll(i)["t_start"] for i in ids]
     assert start[0] < start[2] < start[1]
     srv.close()
+
+
+def test_sixteen_right_hand_sides_next_to_one_another(pkg):
+    """The coefficients of an update are beyond 64 KB from 16 steps of 16 right-hand
+    sides on: their host copy lasts until the device has read it.  The same
+    results in a mix of four as alone."""
+    reqs = []
+    for i, T in enumerate((24, 40, 33, 28, 36, 45, 30, 26)):
+        wl = mi.config1(seed=i, T=T, kappa=9.0 + i, nrhs=16)
+        reqs.append((wl, wl.boundary_data()))
+    got = []
+    for slots in (1, 4):
+        srv = pkg.Server(max_active=slots)
+        ids = [srv.submit(wl, v, tol=1e-9) for wl, v in reqs]
+        srv.drain()
+        res = [srv.poll(rid, want_solution=True) for rid in ids]
+        srv.close()
+        assert all(r["done"] == 1 and r["converged"] == 1 for r in res)
+        assert min(r["inner_iterations"] for r in res) > 16
+        got.append([r["qhat"] for r in res])
+    for a, b in zip(*got):
+        assert np.array_equal(a, b)
