@@ -595,35 +595,36 @@ Shape32 shape32(mbs_ctx* c, int nrhs, const float2* x, float2* y) {
     // The kernel path first, at the usual split counts: the other counts change
     // times by up to a fifth, and what the paths' roundings differ by is not
     // theirs to decide (3D: FP32 pipe 1e-6 off, tensor cores 5e-6).  Then the
-    // counts of that path.  All buffers and each path's first launch come before
-    // its timed ones.
+    // counts of that path.  All buffers come before the timed launches, and a
+    // kernel's first launch, which may load it, counts from 5 ms on only.
     cudaEvent_t a = take_event(c), b = take_event(c);
-    auto time = [&](const Shape32& sh, float stop) {
+    auto once = [&](const Shape32& sh) {
         float ms = 0.f;
-        for (int rep = 0; rep < 3 && (rep == 0 || (ms < 0.2f && ms < stop)); ++rep) {
-            MBS_CUDA_TRY(cudaEventRecord(a, c->st));
-            launch_g32(c, nrhs, x, y, sh, nullptr, nullptr);
-            MBS_CUDA_TRY(cudaEventRecord(b, c->st));
-            MBS_CUDA_TRY(cudaEventSynchronize(b));
-            float t = 0.f;
-            MBS_CUDA_TRY(cudaEventElapsedTime(&t, a, b));
-            ms = rep == 0 ? t : std::min(ms, t);
-        }
+        MBS_CUDA_TRY(cudaEventRecord(a, c->st));
+        launch_g32(c, nrhs, x, y, sh, nullptr, nullptr);
+        MBS_CUDA_TRY(cudaEventRecord(b, c->st));
+        MBS_CUDA_TRY(cudaEventSynchronize(b));
+        MBS_CUDA_TRY(cudaEventElapsedTime(&ms, a, b));
+        return ms;
+    };
+    auto time = [&](const Shape32& sh, float stop, bool first) {
+        float ms = once(sh);
+        if (first && ms < 5.f) ms = once(sh);
+        for (int rep = 1; rep < 3 && ms < 0.2f && ms < stop; ++rep) ms = std::min(ms, once(sh));
         return ms;
     };
     auto clamp = [&](int ns) { return std::max(1, std::min(ns, max_nsplit(c))); };
-    launch_g32(c, nrhs, x, y, h, nullptr, nullptr);
+    prepare_g32(c, nrhs, h);
     const size_t held = c->bufs["part32"].n;
     Shape32 best = h;
-    float best_ms = time(h, HUGE_VALF);
+    float best_ms = time(h, HUGE_VALF, true);
     if (c->opt.mac_path == 0 && h.path == 3) {
         const int base = choose_nsplit(c, c->N);
         Shape32 f{1, base}, g{1, clamp(base / 2)};
         if (fits32(c, nrhs, f)) {
-            launch_g32(c, nrhs, x, y, f, nullptr, nullptr);
-            float ms = time(f, HUGE_VALF);
-            if (g.nsplit != base) {
-                const float t = time(g, 1.25f * ms);
+            float ms = time(f, HUGE_VALF, true);
+            if (g.nsplit != base && ms < 1.25f * best_ms) {  // the half was never a tenth faster
+                const float t = time(g, 1.25f * ms, false);
                 if (t < ms) ms = t, f = g;
             }
             // in 3D the more accurate path of two as fast (11 right-hand sides, FP32
@@ -641,7 +642,7 @@ Shape32 shape32(mbs_ctx* c, int nrhs, const float2* x, float2* y) {
         seen.push_back(ns);
         const Shape32 sh{best.path, ns};
         if (!fits32(c, nrhs, sh)) continue;
-        const float ms = time(sh, 1.25f * best_ms);
+        const float ms = time(sh, 1.25f * best_ms, false);
         if (ms < best_ms) best_ms = ms, best = sh;
     }
     c->ev_pool.push_back(a);
