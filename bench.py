@@ -95,14 +95,14 @@ def parse():
                     help="steps of the end-to-end (host buffers) measurement")
     ap.add_argument("--fp64-max-iter", type=int, default=8000,
                     help="iteration cap of the measured plain-FP64 solve (config 1)")
-    ap.add_argument("--serve-requests", type=int, default=64,
+    ap.add_argument("--serve-requests", type=int, default=5,
                     help="requests of the served trace at full size (0 = skip serving)")
     ap.add_argument("--serve-tmax", type=int, default=3000)
     ap.add_argument("--serve-max-iter", type=int, default=20,
                     help="inner-iteration cap per served request of the full-size trace")
     ap.add_argument("--serve-policy", choices=["fifo", "sjf"], default="sjf",
                     help="admission order of the server: arrival order, or shortest estimated work first")
-    ap.add_argument("--serve-compare", type=int, default=8,
+    ap.add_argument("--serve-compare", type=int, default=4,
                     help="requests of the body-count-20..300 trace served by both the mixed and the FP64 "
                          "path (0 = skip)")
     ap.add_argument("--mac", type=int, default=0,
