@@ -389,7 +389,10 @@ int* split_table(mbs_ctx* c, int ns) {
     }
     sb[ns] = c->T;
     int* d = static_cast<int*>(dalloc(c, sb.size() * sizeof(int)));
-    MBS_CUDA_TRY(cudaMemcpy(d, sb.data(), sb.size() * sizeof(int), cudaMemcpyHostToDevice));
+    // on the stream that reads it: a copy from pageable memory on another one may
+    // still be on its way when the call has returned
+    const Drain drain{c->st};
+    MBS_CUDA_TRY(cudaMemcpyAsync(d, sb.data(), sb.size() * sizeof(int), cudaMemcpyHostToDevice, c->st));
     c->split_cache[key] = d;
     return d;
 }
@@ -2374,18 +2377,19 @@ mbs_status mbs_inject_scattering(mbs_ctx* c, int shape, int k, const int* skel, 
         s.skel.assign(skel, skel + k);
         s.S64 = galloc<double2>(c, (size_t)k * k);
         s.S32 = galloc<float2>(c, (size_t)k * k);
-        MBS_CUDA_TRY(cudaMemcpy(s.S64, S, (size_t)k * k * sizeof(double2), cudaMemcpyHostToDevice));
+        MBS_CUDA_TRY(cudaMemcpyAsync(s.S64, S, (size_t)k * k * sizeof(double2), cudaMemcpyHostToDevice, c->st));
         launch_f64_to_f32(s.S64, s.S32, (int64_t)k * k, c->st);
         double sq = 0.0;
         for (size_t e = 0; e < (size_t)2 * k * k; ++e) sq += S[e] * S[e];
         s.snorm = std::sqrt(sq);
         if (W) {
             s.W = galloc<double2>(c, (size_t)k * s.m);
-            MBS_CUDA_TRY(cudaMemcpy(s.W, W, (size_t)k * s.m * sizeof(double2), cudaMemcpyHostToDevice));
+            MBS_CUDA_TRY(cudaMemcpyAsync(s.W, W, (size_t)k * s.m * sizeof(double2), cudaMemcpyHostToDevice, c->st));
         } else {
             s.W = nullptr;
         }
         c->layout_dirty = true;  // rebuilt by the next call that needs the layout
+        MBS_CUDA_TRY(cudaStreamSynchronize(c->st));  // S and W are the caller's
         return MBS_OK;
     });
 }
