@@ -595,11 +595,13 @@ Shape32 shape32(mbs_ctx* c, int nrhs, const float2* x, float2* y) {
         sh.nsplit = std::min(sh.nsplit, max_nsplit(c));
         return sh;
     }
-    // The kernel path first, at the usual split counts: the other counts change
-    // times by up to a fifth, and what the paths' roundings differ by is not
-    // theirs to decide (3D: FP32 pipe 1e-6 off, tensor cores 5e-6).  Then the
-    // counts of that path.  All buffers come before the timed launches, and a
-    // kernel's first launch, which may load it, counts from 5 ms on only.
+    // 2D: the fastest of all shapes (both paths' roundings are alike: 6e-6 and 6e-6
+    // off on 400 bodies, 4.4e-5 and 5.0e-5 on bodies of uneven size).  3D: the path
+    // at the usual split counts, then the counts of that path, since these change
+    // times by up to a fifth and what the paths' roundings differ by (FP32 pipe 1e-6
+    // off, tensor cores 5e-6) is not theirs to decide.  All buffers come before the
+    // timed launches, and a kernel's first launch, which may load it, counts from
+    // 5 ms on only.
     cudaEvent_t a = take_event(c), b = take_event(c);
     auto once = [&](const Shape32& sh) {
         float ms = 0.f;
@@ -621,33 +623,34 @@ Shape32 shape32(mbs_ctx* c, int nrhs, const float2* x, float2* y) {
     const size_t held = c->bufs["part32"].n;
     Shape32 best = h;
     float best_ms = time(h, HUGE_VALF, true);
-    if (c->opt.mac_path == 0 && h.path == 3) {
-        const int base = choose_nsplit(c, c->N);
-        Shape32 f{1, base}, g{1, clamp(base / 2)};
-        if (fits32(c, nrhs, f)) {
-            float ms = time(f, HUGE_VALF, true);
-            if (g.nsplit != base && ms < 1.25f * best_ms) {  // the half was never a tenth faster
-                const float t = time(g, 1.25f * ms, false);
-                if (t < ms) ms = t, f = g;
-            }
-            // in 3D the more accurate path of two as fast (11 right-hand sides, FP32
-            // pipe and tensor cores: 35 ellipsoids 515 and 509 us, but 19 238 and 213)
-            if (ms < (c->dim == 3 ? 1.03f : 1.f) * best_ms) best_ms = ms, best = f;
+    // half, double and, for tcgen05, four times a path's usual count: small CTAs even
+    // out bodies of uneven size (700 bodies, 16 right-hand sides: 4.64 ms with 14
+    // splits, 4.30 with 28); the FP32-pipe kernel gains nothing from four times
+    auto others = [&](int path, int base) {
+        std::vector<int> seen{base};
+        for (int ns : {clamp(base / 2), clamp(2 * base), clamp(path == 3 ? 4 * base : base)}) {
+            if (std::find(seen.begin(), seen.end(), ns) != seen.end()) continue;
+            seen.push_back(ns);
+            const Shape32 sh{path, ns};
+            if (!fits32(c, nrhs, sh)) continue;
+            float ms = time(sh, 1.25f * best_ms, false);
+            // a narrow loss may be the fresh buffer's: up to 1 ms once more
+            if (ms >= 0.2f && ms < 1.f && ms >= best_ms && ms < 1.05f * best_ms) ms = once(sh);
+            if (ms < best_ms) best_ms = ms, best = sh;
         }
+    };
+    const Shape32 f{1, choose_nsplit(c, c->N)};  // the other path's usual count
+    const bool both = c->opt.mac_path == 0 && h.path == 3, early = c->dim == 2 || !both;
+    if (early) others(h.path, h.nsplit);
+    if (both && fits32(c, nrhs, f)) {
+        const float ms = time(f, HUGE_VALF, true);
+        const bool near = ms < 1.25f * best_ms;  // no count was a fifth faster than the usual one
+        // in 3D the more accurate path of two as fast (11 right-hand sides, FP32
+        // pipe and tensor cores: 35 ellipsoids 515 and 509 us, but 19 238 and 213)
+        if (ms < (c->dim == 3 ? 1.03f : 1.f) * best_ms) best_ms = ms, best = f;
+        if (early && near) others(1, f.nsplit);
     }
-    // four times the usual count: small CTAs even out bodies of uneven size (700
-    // bodies, 16 right-hand sides: 4.64 ms with 14 splits, 4.30 with 28); the
-    // FP32-pipe kernel gains nothing
-    const int base = best.path == 3 ? h.nsplit : choose_nsplit(c, c->N);
-    std::vector<int> seen{base, best.path == 1 && h.path == 3 ? clamp(base / 2) : base};
-    for (int ns : {clamp(base / 2), clamp(2 * base), clamp(best.path == 3 ? 4 * base : base)}) {
-        if (std::find(seen.begin(), seen.end(), ns) != seen.end()) continue;
-        seen.push_back(ns);
-        const Shape32 sh{best.path, ns};
-        if (!fits32(c, nrhs, sh)) continue;
-        const float ms = time(sh, 1.25f * best_ms, false);
-        if (ms < best_ms) best_ms = ms, best = sh;
-    }
+    if (!early) others(best.path, best.nsplit);
     c->ev_pool.push_back(a);
     c->ev_pool.push_back(b);
     // partial sums beyond what the fastest shape needs go back
