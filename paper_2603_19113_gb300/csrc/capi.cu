@@ -455,8 +455,8 @@ int* device_err(mbs_ctx* c) {
 // problem class (device, dimension, right-hand sides, kernel option and the
 // power-of-two buckets of N and of the body count) times every candidate
 // shape on the caller's own data: the kernel path (tcgen05 or FP32 pipe,
-// unless mac_path fixes it), then the source-split count (the heuristic's,
-// half, double and four times it).  The fastest is kept in a process-wide table, so every
+// unless mac_path fixes it) with the source-split counts (the heuristic's,
+// half, double and, for tcgen05, four times it).  The fastest is kept in a process-wide table, so every
 // later matvec of that class, in any context, uses the same shape; a solve
 // therefore gives the same result alone and next to other solves.
 // mbs_options.autotune = 0 (or a tile_override) keeps the heuristic shape.
@@ -595,13 +595,11 @@ Shape32 shape32(mbs_ctx* c, int nrhs, const float2* x, float2* y) {
         sh.nsplit = std::min(sh.nsplit, max_nsplit(c));
         return sh;
     }
-    // 2D: the fastest of all shapes (both paths' roundings are alike: 6e-6 and 6e-6
-    // off on 400 bodies, 4.4e-5 and 5.0e-5 on bodies of uneven size).  3D: the path
-    // at the usual split counts, then the counts of that path, since these change
-    // times by up to a fifth and what the paths' roundings differ by (FP32 pipe 1e-6
-    // off, tensor cores 5e-6) is not theirs to decide.  All buffers come before the
-    // timed launches, and a kernel's first launch, which may load it, counts from
-    // 5 ms on only.
+    // The fastest of all shapes, but in 3D the FP32 pipe where it is about as fast:
+    // its sums are 1e-6 off, the tensor cores' 5e-6 (in 2D they are alike: 6e-6 both
+    // on 400 bodies, 4.4e-5 and 5.0e-5 on bodies of uneven size).  All buffers come
+    // before the timed launches, and a kernel's first launch, which may load it,
+    // counts from 5 ms on only.
     cudaEvent_t a = take_event(c), b = take_event(c);
     auto once = [&](const Shape32& sh) {
         float ms = 0.f;
@@ -623,15 +621,13 @@ Shape32 shape32(mbs_ctx* c, int nrhs, const float2* x, float2* y) {
     const size_t held = c->bufs["part32"].n;
     Shape32 best = h;
     float best_ms = time(h, HUGE_VALF, true);
-    // half, double and, for tcgen05, four times a path's usual count: small CTAs even
-    // out bodies of uneven size (700 bodies, 16 right-hand sides: 4.64 ms with 14
-    // splits, 4.30 with 28); the FP32-pipe kernel gains nothing from four times
-    auto others = [&](int path, int base) {
-        std::vector<int> seen{base};
-        for (int ns : {clamp(base / 2), clamp(2 * base), clamp(path == 3 ? 4 * base : base)}) {
-            if (std::find(seen.begin(), seen.end(), ns) != seen.end()) continue;
-            seen.push_back(ns);
-            const Shape32 sh{path, ns};
+    std::vector<Shape32> seen{h};
+    auto others = [&](int path, std::initializer_list<int> counts, Shape32& best, float& best_ms) {
+        for (int ns : counts) {
+            const Shape32 sh{path, clamp(ns)};
+            if (std::any_of(seen.begin(), seen.end(), [&](const Shape32& q) { return q.path == path && q.nsplit == sh.nsplit; }))
+                continue;
+            seen.push_back(sh);
             if (!fits32(c, nrhs, sh)) continue;
             float ms = time(sh, 1.25f * best_ms, false);
             // a narrow loss may be the fresh buffer's: up to 1 ms once more
@@ -639,18 +635,25 @@ Shape32 shape32(mbs_ctx* c, int nrhs, const float2* x, float2* y) {
             if (ms < best_ms) best_ms = ms, best = sh;
         }
     };
-    const Shape32 f{1, choose_nsplit(c, c->N)};  // the other path's usual count
-    const bool both = c->opt.mac_path == 0 && h.path == 3, early = c->dim == 2 || !both;
-    if (early) others(h.path, h.nsplit);
-    if (both && fits32(c, nrhs, f)) {
-        const float ms = time(f, HUGE_VALF, true);
-        const bool near = ms < 1.25f * best_ms;  // no count was a fifth faster than the usual one
-        // in 3D the more accurate path of two as fast (11 right-hand sides, FP32
-        // pipe and tensor cores: 35 ellipsoids 515 and 509 us, but 19 238 and 213)
-        if (ms < (c->dim == 3 ? 1.03f : 1.f) * best_ms) best_ms = ms, best = f;
-        if (early && near) others(1, f.nsplit);
+    const int b3 = h.nsplit, b1 = choose_nsplit(c, c->N);
+    const float usual_ms = best_ms;
+    others(h.path, {b3 / 2, 2 * b3}, best, best_ms);
+    bool pipe = false;  // the FP32 pipe instead of tcgen05
+    Shape32 f{1, b1};
+    if (c->opt.mac_path == 0 && h.path == 3 && fits32(c, nrhs, f)) {
+        seen.push_back(f);
+        float ms = time(f, HUGE_VALF, true);
+        // 3D: within 3 % at the usual counts or 6 % at the best (FP32 pipe and tensor
+        // cores: 11 right-hand sides, 35 ellipsoids 515 and 509 us, but 19 238 and 213;
+        // 4, 57 ellipsoids 511 and 492 at the usual, 456 and 470 at the best)
+        pipe = c->dim == 3 && ms < 1.03f * usual_ms;
+        if (pipe || ms < 1.25f * best_ms) others(1, {b1 / 2, 2 * b1}, f, ms);  // no count was a fifth faster
+        pipe = pipe || ms < (c->dim == 3 ? 1.06f : 1.f) * best_ms;
+        if (pipe) best_ms = ms, best = f;
     }
-    if (!early) others(best.path, best.nsplit);
+    // four times: small CTAs even out bodies of uneven size (700 bodies, 16 right-hand
+    // sides: 4.64 ms with 14 splits, 4.30 with 28); the FP32-pipe kernel gains nothing
+    if (h.path == 3 && !(pipe && c->dim == 3)) others(3, {4 * b3}, best, best_ms);
     c->ev_pool.push_back(a);
     c->ev_pool.push_back(b);
     // partial sums beyond what the fastest shape needs go back
